@@ -319,7 +319,9 @@ def kernel_models(plan, grid, sprec, fprec):
         fl_band = sum((n - w) * w * (w + 1) + 2.0 * n for n, w in narrow if w <= 12)
         m.update({"k_f32_shadow_in": (band_lo * 16.0, 0.0, fprec), "k_f32_out": ((band_lo + l21_lo) * 16.0, 0.0, fprec),
                   "k_f64_band_pass": (band_lo * 16.0, fl_band, "fp64"),
-                  "k_df_band_pass": (band_lo * 16.0, fl_band, "fp32x2")})
+                  "k_df_band_pass": (band_lo * 16.0, fl_band, "fp32x2"),
+                  "k_f64_window": (b12, fl12, "fp64"),
+                  "k_df_window": (b12, fl12, "fp32x2")})
         for name in ("k_l21_transfer", "k_l21_carry", "k_l21_solve", "k_l21_cornerpart", "k_l21_corner"):
             m[name] = (0.0, None, fprec, "a phase of the chunked border solve, not modelled alone")
         return m

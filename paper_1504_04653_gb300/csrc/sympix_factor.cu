@@ -57,7 +57,9 @@ extern "C" int sympix_factor_blocks(sympix_plan_t pl, int storage, int precision
     // kernels for every w <= 16
     const bool narrow = !dense && pl->narrow_pref[precision] == 0;
     if (narrow) launch_pband_chol(pl, precision, blocks, info, st);
-    if (precision == SYMPIX_PREC_FP64 && !dense && pl->narrow_pref[precision] == 2) {
+    if (precision != SYMPIX_PREC_FP32 && !dense && pl->narrow_pref[precision] == kNarrowWindow) {
+        launch_window(pl, precision, blocks, info, st);  // w <= 12 in one pass, lane groups above
+    } else if (precision == SYMPIX_PREC_FP64 && !dense && pl->narrow_pref[precision] == 2) {
         launch_f64_slices(pl, blocks, info, st);  // w <= 12 on the FP64 shadow, lane groups above
     } else if (precision == SYMPIX_PREC_FP32X2 && !dense && pl->narrow_pref[precision] == 2) {
         launch_df_slices(pl, blocks, info, st);  // w <= 12 on a split-FP32 shadow, lane groups above

@@ -1040,6 +1040,11 @@ void launch_df_l21(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t
 // shadow of that arithmetic (sympix_factor_f32.cu)
 void launch_f64_slices(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st);
 void launch_df_slices(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st);
+// the FP64 / split-FP32 factor of the periodic bands up to w = 16 by the
+// sliding-window kernel (sympix_window.cuh) and the lane groups
+void launch_window(sympix_plan_t pl, int precision, double *blocks, int32_t *info, cudaStream_t st);
+void launch_window_f64(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st);
+void launch_window_df(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st);
 constexpr int kDefaultWaitLimit = 1 << 22;  // polls of a bounded device wait (about 0.3 s)
 void launch_factor_wide_dense(sympix_plan_t pl, int precision, bool dense, double *blocks, int32_t *info,
                               cudaStream_t st);

@@ -57,6 +57,8 @@ bool f32_split_fits(sympix_plan_t pl);
 // Widest band of the narrow-band factor (k_pband_chol), and the elements of
 // one tile of its FP32 commit.
 constexpr int kNarrowWMax = 12;
+// narrow_pref of the sliding-window kernel (FP64 and split FP32)
+constexpr int kNarrowWindow = 4;
 constexpr int kCommitTileElems = 2048;
 
 // Smallest relative distance |u - u_s| / u_s a support class may have from
@@ -318,6 +320,12 @@ struct sympix_plan_s {
     std::vector<CholSlice> chol_sl32, chol_sl64;
     std::vector<int2> chol_tiles;
     int chol_wmax = -1;
+    // sliding-window factor (FP64 and split FP32): one warp per entry (first
+    // of chol_items, count, width), longest first; [0] as many blocks per
+    // warp as the width allows, [1] one block per warp, and which list each
+    // arithmetic runs
+    sympix::DevBuf<int4> d_win[2];
+    int win_one[3] = {0, 0, 0};
     // per width: the slices [chol_f32[w], + chol_n32[w]) of chol_sl32 and
     // [chol_f64[w], + chol_n64[w]) of chol_sl64; a stream per width present
     // (the widths run side by side) and the fork / join events
@@ -332,10 +340,8 @@ struct sympix_plan_s {
     // two-role kernel on an FP32 band copy; FP64 / split FP32: lane groups),
     // 2 band pass and chunked border solve on a shadow of the arithmetic,
     // 3 (FP32) band and border CTAs of one cooperative launch for w <= 8, 2
-    // for 9 <= w <= 12.  Defaults from measurement at l_max = 3000 (factor
-    // stage): FP64 2 (12.9 ms; 0: 20.1 ms), FP32 3, split FP32 2 (6.0 ms;
-    // 1: 30.2 ms).
-    int narrow_pref[3] = {2, 3, 2};
+    // for 9 <= w <= 12, kNarrowWindow (FP64 and split FP32) the sliding window.
+    int narrow_pref[3] = {sympix::kNarrowWindow, 3, sympix::kNarrowWindow};
     // DP-grid plans (k > 1): band blocks under tile adjacency
     bool tiles = false;
     std::vector<TileBlock> tile_blocks;

@@ -16,7 +16,7 @@
 #include <numeric>
 #include <unordered_map>
 
-#include "sympix_internal.cuh"
+#include "sympix_window.cuh"
 
 namespace sympix {
 
@@ -544,6 +544,33 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
             }
         }
     }
+    // sliding-window factor: warps of both layouts, longest first, and the
+    // layout whose estimated time (the longest warp, or all of them spread
+    // over the schedulers) is shorter
+    {
+        double est[2] = {0.0, 0.0};
+        for (int one = 0; one < 2; ++one) {
+            std::vector<std::pair<double, int4>> work;
+            double total = 0.0, longest = 0.0;
+            for (size_t i = 0; i < pl->chol_items.size();) {
+                const int w = pl->blocks[pl->chol_items[i]].w;
+                const int per = one ? 1 : 32 / window_rows(w);
+                size_t e = i;
+                while (e < pl->chol_items.size() && e < i + per && pl->blocks[pl->chol_items[e]].w == w) ++e;
+                const double cost = window_step_cost(w, 32 / per) * pl->blocks[pl->chol_items[i]].n;
+                work.push_back({cost, make_int4((int)i, (int)(e - i), w, 0)});
+                total += cost;
+                longest = std::max(longest, cost);
+                i = e;
+            }
+            std::stable_sort(work.begin(), work.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
+            std::vector<int4> list;
+            for (const auto &x : work) list.push_back(x.second);
+            if ((rc = pl->d_win[one].upload(list))) return fail(rc);
+            est[one] = std::max(longest, total / 608.0);
+        }
+        for (int &o : pl->win_one) o = est[1] < est[0] ? 1 : 0;
+    }
     // chunked border solve of the fused-range slices (1 <= w <= 12)
     pl->l21_first.assign(pl->f32_slices_fused, -1);
     pl->l21_nch.assign(pl->f32_slices_fused, 0);
@@ -643,9 +670,9 @@ extern "C" int sympix_plan_option(sympix_plan_t pl, int option, double value) {
         if (value != 0.0 && value != 1.0 && value != 2.0 && value != 3.0 && value != -1.0)
             return set_error(SYMPIX_EINVAL, "sympix_plan_option: narrow factor kernel is -1, 0, 1, 2 or 3");
         if (value == -1.0) {
-            pl->narrow_pref[SYMPIX_PREC_FP64] = 2;
+            pl->narrow_pref[SYMPIX_PREC_FP64] = kNarrowWindow;
             pl->narrow_pref[SYMPIX_PREC_FP32] = 3;
-            pl->narrow_pref[SYMPIX_PREC_FP32X2] = 2;
+            pl->narrow_pref[SYMPIX_PREC_FP32X2] = kNarrowWindow;
         } else if (value == 2.0 || value == 3.0) {
             // the chunked border solve (every arithmetic) and the split kernel (FP32)
             pl->narrow_pref[SYMPIX_PREC_FP64] = 2;
@@ -691,7 +718,7 @@ extern "C" int sympix_plan_tuning(sympix_plan_t pl, int *table_cta, int *border_
     if (table_cta) *table_cta = pl->table_cta;
     if (border_threads) *border_threads = pl->border_threads;
     if (narrow)
-        for (int i = 0; i < 3; ++i) narrow[i] = pl->narrow_pref[i];
+        for (int i = 0; i < 3; ++i) narrow[i] = pl->narrow_pref[i] == kNarrowWindow ? 2 : pl->narrow_pref[i];
     return SYMPIX_OK;
 }
 
@@ -738,8 +765,8 @@ extern "C" int sympix_autotune(sympix_plan_t pl, const double *bl, const double 
         factor_precision <= 2) {
         best = 1e30f;
         int best_k = pl->narrow_pref[factor_precision];
-        for (int kk : {0, 1, 2, 3}) {
-            if (kk == 3 && factor_precision != SYMPIX_PREC_FP32) continue;
+        for (int kk : {0, 1, 2, 3, kNarrowWindow}) {
+            if (kk == (factor_precision == SYMPIX_PREC_FP32 ? kNarrowWindow : 3)) continue;
             pl->narrow_pref[factor_precision] = kk;
             float ms = 0.0f;
             auto run = [&] {
@@ -869,6 +896,9 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
         }
     } else if (factor_precision == SYMPIX_PREC_FP32) {
         f += (l0 || l1 || l2) ? 2 : 0;  // both passes for every width up to 16
+    } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == kNarrowWindow) {
+        // w <= 12 in the sliding-window kernel, then the lane groups of 12 < w <= 16
+        f += (pl->chol_items.empty() ? 0 : 1) + (l2 ? 1 : 0);
     } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == 2) {
         // w <= 12 on the FP64 / split-FP32 shadow: transpose in, band pass, transfer, carry,
         // solve and corner sums of each width range, corners, write-back; then
