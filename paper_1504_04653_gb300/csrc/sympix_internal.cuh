@@ -36,6 +36,8 @@ void trace_mark(sympix_plan_t pl, cudaStream_t st, const char *name);
 long tile_pair_mmax(int na, int nb, int k, bool all);
 int plan_tile_blocks(sympix_plan_t pl, const std::unordered_map<int64_t, int> &index, int g0, int g1);
 int launch_tiles(sympix_plan_t pl, const double *ninv, int precision, double *blocks, cudaStream_t st);
+// Work lists of sympix_apply (sympix_apply.cu); `order`: blocks, most expensive first.
+int plan_apply(sympix_plan_t pl, const std::vector<int32_t> &order);
 inline std::pair<int, int> canon_pair(int N, int j, int rho) {
     int a = j < rho ? j : rho, b = j < rho ? rho : j;
     if (a > N - 1 - b) {
@@ -383,6 +385,14 @@ struct sympix_plan_s {
     // class (not only the same-ring ones) once such a layout exists
     std::map<int, CouplingPlan> coupling;
     bool all_d = false, table_all_d = false;
+    // the block preconditioner on periodic-band storage (sympix_apply.cu): its
+    // blocks, one warp per work entry (first of the items, count, width; -1: a
+    // dense-format block) in both layouts, and the blocks left to k_apply
+    std::vector<int4> apply_work[2];
+    sympix::DevBuf<int4> d_apply_work[2];
+    sympix::DevBuf<int32_t> d_apply_items, d_apply_rest;
+    int apply_rest = 0;
+    bool apply_one = false;
     sympix::DevBuf<int64_t> d_ring_off;  // the grid's ring offsets and strides (the apply's pixel addresses)
     sympix::DevBuf<int32_t> d_ring_stride;
     // tracing (SYMPIX_OPT_TRACE): an event after every launch of a traced

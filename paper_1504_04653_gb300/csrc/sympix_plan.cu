@@ -400,6 +400,7 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
         return bd.format == SYMPIX_BLOCK_PBAND ? n * (w + 1) * (3 * w + 1) : n * n * n / 3.0;
     };
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
+    if (!tiles && (rc = plan_apply(pl, order))) return fail(rc);
     for (int b : order) {
         const BlockDesc &bd = pl->blocks[b];
         int list;

@@ -130,6 +130,13 @@ __host__ __device__ constexpr int window_elems(int W, int G) {
     return (kWindowPeriods * W * (W + 1) + W * (2 * G + 1) + W * W + 2 * G + 2 + 1) / 2 * 2;
 }
 
+// The block preconditioner on periodic bands (sympix_apply.cu): the widest
+// band, lanes per block of a full warp, and one block's shared memory (doubles:
+// four periods of band rows, the corner).
+constexpr int kApplyWMax = 16;
+__host__ __device__ constexpr int apply_lanes(int W) { return W <= 8 ? 8 : 16; }
+__host__ __device__ constexpr int apply_elems(int W) { return (4 * W * (W + 1) + W * W + 1) / 2 * 2; }
+
 // Sums of acc over the G lanes of a group: each exchange adds the halves of
 // two lanes' arrays, so lane l ends with sums at, at + 1, ... of its own.
 template <class V, int N, int O>
