@@ -256,7 +256,12 @@ struct CoupDesc {
 struct CouplingPlan {
     std::vector<CoupDesc> desc;
     int64_t total = 0;  // stored entries
-    sympix::DevBuf<CoupDesc> d_desc;
+    // blocks of k_sample_coupling_arcs with their first tiles, and the others
+    // with their first entries among the total_rest
+    int64_t tiles = 0, total_rest = 0;
+    sympix::DevBuf<CoupDesc> d_arcs, d_rest;
+    sympix::DevBuf<int32_t> d_tile0;
+    sympix::DevBuf<int64_t> d_first;
 };
 
 struct sympix_plan_s {

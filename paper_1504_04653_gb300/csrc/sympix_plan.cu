@@ -979,7 +979,10 @@ extern "C" int sympix_plan_device_bytes(sympix_plan_t pl, size_t *bytes, size_t 
                pl->d_l21_slices.bytes() + pl->d_l21_first.bytes() + pl->d_l21_nch.bytes() + pl->d_l21_T.bytes() +
                pl->d_l21_P.bytes() + pl->d_l21_S.bytes() + pl->d_l21_C.bytes() + pl->d_split_flags.bytes() +
                pl->d_split_bandres.bytes() + pl->d_f32_tiles_lo.bytes() + pl->d_f32_out_tiles_lo.bytes();
-    for (const auto &kv : pl->coupling) b += kv.second.d_desc.bytes();
+    for (const auto &kv : pl->coupling)
+        b += kv.second.d_arcs.bytes() + kv.second.d_rest.bytes() + kv.second.d_tile0.bytes() + kv.second.d_first.bytes();
+    b += pl->d_apply_items.bytes() + pl->d_apply_rest.bytes();
+    for (int i = 0; i < 2; ++i) b += pl->d_win[i].bytes() + pl->d_apply_work[i].bytes();
     for (int i = 0; i < 5; ++i) b += pl->d_items_pband[i].bytes();
     for (int i = 0; i < 6; ++i) b += pl->d_factor_items[i].bytes();
     if (bytes) *bytes = b;
