@@ -281,6 +281,8 @@ struct sympix_plan_s {
     int max_w = 0;
     // sampling schedule (built once)
     std::vector<SampleItem> items_pband[5];  // buckets of WMAX = 8,16,32,64,128
+    std::vector<SampleItem> items_wide[3];  // FP32, bands of 17 .. 31, 32 .. 47, 48 .. 64 (sympix_sample_wide.cu)
+    int wide_list_w[3] = {0, 0, 0};         // widest band of each
     std::vector<SampleItem> items_dense;       // dense-format blocks with n <= 64: a warp per element
     std::vector<SampleItem> items_dense_rows;  // larger ones: a thread per element, 256 per CTA
     std::vector<ConvItem> items_conv;  // every block in tiles of 128 pixels
@@ -372,7 +374,7 @@ struct sympix_plan_s {
     sympix::DevBuf<BlockDesc> d_blocks;
     sympix::DevBuf<PairEntry> d_entries;
     sympix::DevBuf<SampleItem> d_items_pband[5];
-    sympix::DevBuf<SampleItem> d_items_dense, d_items_dense_rows;
+    sympix::DevBuf<SampleItem> d_items_dense, d_items_dense_rows, d_items_wide[3];
     sympix::DevBuf<ConvItem> d_items_conv;
     sympix::DevBuf<int32_t> d_factor_items[6];
     sympix::DevBuf<int32_t> d_f32_items;

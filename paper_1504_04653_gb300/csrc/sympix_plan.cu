@@ -377,6 +377,11 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
         if (bd.format == SYMPIX_BLOCK_PBAND) {
             int bucket = bd.w <= 8 ? 0 : bd.w <= 16 ? 1 : bd.w <= 32 ? 2 : 3;
             for (int q0 = 0; q0 < bd.n; q0 += 128) pl->items_pband[bucket].push_back({(int32_t)b, q0});
+            if (bd.w > 16) {
+                const int list = bd.w <= 31 ? 0 : bd.w <= 47 ? 1 : 2;
+                for (int q0 = 0; q0 < bd.n; q0 += 128) pl->items_wide[list].push_back({(int32_t)b, q0});
+                pl->wide_list_w[list] = std::max(pl->wide_list_w[list], bd.w);
+            }
         } else {
             const int64_t ne = (int64_t)bd.n * bd.n;
             if (bd.n <= 64)
@@ -625,6 +630,8 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
         return fail(rc);
     for (int bkt = 0; bkt < 5; ++bkt)
         if ((rc = pl->d_items_pband[bkt].upload(pl->items_pband[bkt]))) return fail(rc);
+    for (int l = 0; l < 3; ++l)
+        if ((rc = pl->d_items_wide[l].upload(pl->items_wide[l]))) return fail(rc);
     for (int l = 0; l < 6; ++l)
         if ((rc = pl->d_factor_items[l].upload(pl->factor_items[l]))) return fail(rc);
     if ((rc = pl->d_status.alloc(1)) || (rc = pl->d_ring_off.upload(grid->offset)) ||
@@ -850,7 +857,12 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
     }
     int s = sample_precision != SYMPIX_PREC_FP64 ? 1 : 0;  // the N^-1 split
     s += pl->tile_items.empty() ? 0 : 1;                     // band blocks of a DP grid
-    for (int b = 0; b < 4; ++b) s += pl->items_pband[b].empty() ? 0 : 1;
+    if (sample_precision == SYMPIX_PREC_FP32 && storage == SYMPIX_STORE_PBAND) {  // w <= 16, then the wide lists
+        for (int b = 0; b < 2; ++b) s += pl->items_pband[b].empty() ? 0 : 1;
+        for (int l = 0; l < 3; ++l) s += pl->items_wide[l].empty() ? 0 : 1;
+    } else {
+        for (int b = 0; b < 4; ++b) s += pl->items_pband[b].empty() ? 0 : 1;
+    }
     s += pl->items_dense.empty() ? 0 : 1;
     s += pl->items_dense_rows.empty() ? 0 : 1;
     if (sample) *sample = s;
@@ -984,6 +996,7 @@ extern "C" int sympix_plan_device_bytes(sympix_plan_t pl, size_t *bytes, size_t 
     b += pl->d_apply_items.bytes() + pl->d_apply_rest.bytes();
     for (int i = 0; i < 2; ++i) b += pl->d_win[i].bytes() + pl->d_apply_work[i].bytes();
     for (int i = 0; i < 5; ++i) b += pl->d_items_pband[i].bytes();
+    for (int i = 0; i < 3; ++i) b += pl->d_items_wide[i].bytes();
     for (int i = 0; i < 6; ++i) b += pl->d_factor_items[i].bytes();
     if (bytes) *bytes = b;
     if (staging) *staging = pl->d_rec.bytes();

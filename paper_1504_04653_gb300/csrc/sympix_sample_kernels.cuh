@@ -412,6 +412,9 @@ __global__ void __launch_bounds__(64) k_sample_pband_f32x2(const SampleItem *__r
     for (int i = threadIdx.x; i < tot; i += 64) dst[i] = stage[i];
 }
 
+// FP32 periodic bands wider than 16 (sympix_sample_wide.cu)
+void launch_sample_wide32(sympix_plan_t pl, double *blocks, cudaStream_t st);
+
 template <int PREC, bool DENSE_OUT>
 void launch_pband(sympix_plan_t pl, const double *ninv, double *blocks, cudaStream_t st) {
     const int64_t npix = pl->grid->npix;
@@ -428,6 +431,7 @@ void launch_pband(sympix_plan_t pl, const double *ninv, double *blocks, cudaStre
                                             pl->d_tab_b32.p, pl->d_tab_d32.p, pl->d_ninv32.p, blocks);
             continue;
         }
+        if (PREC == 1 && !DENSE_OUT && wm[b] > 16) continue;  // below
         // wide bands: the arc-weight cache, kArcCache values per thread
         const size_t wcs = (size_t)128 * kArcCache * sizeof(typename Arith<PREC>::V);
         switch (wm[b]) {
@@ -446,6 +450,7 @@ void launch_pband(sympix_plan_t pl, const double *ninv, double *blocks, cudaStre
         }
 #undef SPX_ARGS
     }
+    if (PREC == 1 && !DENSE_OUT) launch_sample_wide32(pl, blocks, st);
 }
 
 }  // namespace sympix
