@@ -67,9 +67,6 @@ constexpr int kCommitTileElems = 2048;
 // the coupling threshold before the radius is scaled by (1 - 1e-9).
 constexpr double kSupportMargin = 1e-12;
 
-// Elements of a dense-format block sampled by one CTA (a warp each).
-constexpr int kDenseItemElems = 8;
-
 // Elements per block in one CTA of the FP32 shadow transposes (x 32 blocks).
 constexpr int kTileE = 128;
 
@@ -283,8 +280,7 @@ struct sympix_plan_s {
     std::vector<SampleItem> items_pband[5];  // buckets of WMAX = 8,16,32,64,128
     std::vector<SampleItem> items_wide[3];  // FP32, bands of 17 .. 31, 32 .. 47, 48 .. 64 (sympix_sample_wide.cu)
     int wide_list_w[3] = {0, 0, 0};         // widest band of each
-    std::vector<SampleItem> items_dense;       // dense-format blocks with n <= 64: a warp per element
-    std::vector<SampleItem> items_dense_rows;  // larger ones: a thread per element, 256 per CTA
+    std::vector<SampleItem> items_dense;    // dense-format blocks: a row by up to 64 columns
     std::vector<ConvItem> items_conv;  // every block in tiles of 128 pixels
     // factorisation work lists, each most expensive first: periodic band with
     // [0] w <= 8, [1] 8 < w <= 12, [2] 12 < w <= 16, [5] 16 < w <= 64;
@@ -374,7 +370,7 @@ struct sympix_plan_s {
     sympix::DevBuf<BlockDesc> d_blocks;
     sympix::DevBuf<PairEntry> d_entries;
     sympix::DevBuf<SampleItem> d_items_pband[5];
-    sympix::DevBuf<SampleItem> d_items_dense, d_items_dense_rows, d_items_wide[3];
+    sympix::DevBuf<SampleItem> d_items_dense, d_items_wide[3];
     sympix::DevBuf<ConvItem> d_items_conv;
     sympix::DevBuf<int32_t> d_factor_items[6];
     sympix::DevBuf<int32_t> d_f32_items;

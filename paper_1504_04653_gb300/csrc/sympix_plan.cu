@@ -370,8 +370,8 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
     }
 
     // sampling work items: pband blocks in tiles of 128 columns, bucketed by
-    // band width; dense blocks of up to 64 pixels in tiles of 8 elements (a
-    // warp each), larger ones in tiles of 256 (a thread each)
+    // band width; dense blocks as rows q of up to 64 columns r <= q (q0 = q and
+    // the column tile in the high half)
     for (size_t b = 0; b < (tiles ? 0 : pl->blocks.size()); ++b) {
         const BlockDesc &bd = pl->blocks[b];
         if (bd.format == SYMPIX_BLOCK_PBAND) {
@@ -383,11 +383,8 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
                 pl->wide_list_w[list] = std::max(pl->wide_list_w[list], bd.w);
             }
         } else {
-            const int64_t ne = (int64_t)bd.n * bd.n;
-            if (bd.n <= 64)
-                for (int64_t e0 = 0; e0 < ne; e0 += kDenseItemElems) pl->items_dense.push_back({(int32_t)b, (int32_t)e0});
-            else
-                for (int64_t e0 = 0; e0 < ne; e0 += 256) pl->items_dense_rows.push_back({(int32_t)b, (int32_t)e0});
+            for (int q = 0; q < bd.n; ++q)
+                for (int c = 0; 64 * c <= q; ++c) pl->items_dense.push_back({(int32_t)b, q | c << 16});
         }
     }
     // convolution work items: every block's ring in tiles of 128 pixels
@@ -626,7 +623,7 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
                   (rc = pl->d_tile_slot0.upload(pl->tile_slot0)) || (rc = pl->d_tile_noff.upload(pl->tile_noff))))
         return fail(rc);
     if ((rc = pl->d_blocks.upload(pl->blocks)) || (rc = pl->d_entries.upload(pl->entries)) ||
-        (rc = pl->d_items_dense.upload(pl->items_dense)) || (rc = pl->d_items_dense_rows.upload(pl->items_dense_rows)) || (rc = pl->d_items_conv.upload(pl->items_conv)))
+        (rc = pl->d_items_dense.upload(pl->items_dense)) || (rc = pl->d_items_conv.upload(pl->items_conv)))
         return fail(rc);
     for (int bkt = 0; bkt < 5; ++bkt)
         if ((rc = pl->d_items_pband[bkt].upload(pl->items_pband[bkt]))) return fail(rc);
@@ -864,7 +861,6 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
         for (int b = 0; b < 4; ++b) s += pl->items_pband[b].empty() ? 0 : 1;
     }
     s += pl->items_dense.empty() ? 0 : 1;
-    s += pl->items_dense_rows.empty() ? 0 : 1;
     if (sample) *sample = s;
     // mirrors the launch sequence of sympix_factor_blocks
     int f = 0;
@@ -982,7 +978,7 @@ extern "C" int sympix_plan_device_bytes(sympix_plan_t pl, size_t *bytes, size_t 
                pl->d_tab_d.bytes() + pl->d_tab_b32.bytes() + pl->d_tab_blo.bytes() + pl->d_tab_d32.bytes() +
                pl->d_tab_dlo.bytes() + pl->d_ninv32.bytes() + pl->d_ninvlo.bytes() + pl->d_rec.bytes() +
                pl->d_blocks.bytes() + pl->d_entries.bytes() + pl->d_items_dense.bytes() +
-               pl->d_items_dense_rows.bytes() + pl->d_items_conv.bytes() + pl->d_f32_items.bytes() +
+               pl->d_items_conv.bytes() + pl->d_f32_items.bytes() +
                pl->d_f32_slices.bytes() + pl->d_f32_tiles.bytes() + pl->d_shadow_il.bytes() +
                pl->d_l21_il.bytes() + pl->d_f32_out_tiles.bytes() + pl->d_shadow.bytes() + pl->d_chol_items.bytes() +
                pl->d_chol_sl32.bytes() + pl->d_chol_sl64.bytes() + pl->d_chol_tiles.bytes() +

@@ -35,20 +35,31 @@ __global__ void k_split_ninv(int64_t count, const double *__restrict__ ninv, flo
 }
 
 // z reduced to (-half, half] (T2 = 2 half): the longitude separation index
-// of a pixel pair on a pair of rings, as the kernel table is indexed.
-__device__ __forceinline__ int64_t wrap_half(int64_t z, int64_t half, int64_t T2) {
+// of a pixel pair on a pair of rings, as the kernel table is indexed.  Dense
+// blocks have at most 8192 pixels and rings 30000, so that every index and
+// T2 = 2 P n_rho fit 32 bits.
+__device__ __forceinline__ int wrap_half(int z, int half, int T2) {
     z %= T2;
     if (z > half) z -= T2;
     if (z <= -half) z += T2;
     return z;
 }
 
-// Small or wrapping blocks (every pixel pair of the ring may couple): one
-// warp per element (q, r), its lanes sharing the pixels coupled to q on
-// every coupled ring (the arc |z_q| <= mmax, or the whole ring when the
-// support covers it), separation indices reduced to |dphi| <= pi; the
-// partial sums meet in a fixed-order shuffle tree.  FP64.
-__global__ void __launch_bounds__(32 * kDenseItemElems) k_sample_dense(const SampleItem *__restrict__ items,
+// Small or wrapping blocks (every pixel pair of the ring may couple), FP64.
+// A CTA takes row q and up to 64 columns r <= q (M is symmetric: (r, q) is
+// stored with (q, r)).  For eight neighbour rings at a time each of its eight
+// warps forms one ring's weights b(q, p) N^-1_p over the pixels coupled to q
+// (the arc |z_q| <= mmax, or the whole ring when the support covers it),
+// kDensePix at a time; then warp k sums over them for the columns r = k, k + 8,
+// ..., its lanes sharing the pixels, separation indices reduced to |dphi| <=
+// pi and moved by a fixed step.  The partial sums meet in a fixed-order
+// shuffle tree.  Bound by the FP64 pipe and the integer work per pixel: one
+// multiply-add a pixel, half the pairs, against a product and a multiply-add
+// for every (q, r) in 64-bit index arithmetic before (72 blocks of up to 128
+// pixels at l_max 1000: 2.0 -> 0.35 ms).
+constexpr int kDensePix = 256, kDenseWarps = 8, kDenseCols = 64;
+
+__global__ void __launch_bounds__(32 * kDenseWarps) k_sample_dense(const SampleItem *__restrict__ items,
                                                                    const BlockDesc *__restrict__ blocks,
                                                                    const PairEntry *__restrict__ entries,
                                                                    int64_t nslots, int64_t npix,
@@ -56,109 +67,93 @@ __global__ void __launch_bounds__(32 * kDenseItemElems) k_sample_dense(const Sam
                                                                    const double *__restrict__ td,
                                                                    const double *__restrict__ ninv,
                                                                    double *__restrict__ out, int dense_storage) {
+    constexpr int NR = kDenseCols / kDenseWarps;
+    __shared__ double wgt[kDenseWarps][kDensePix];
+    __shared__ int s_len[kDenseWarps], s_pm[kDenseWarps];
     const SampleItem it = items[blockIdx.x];
     const BlockDesc bd = blocks[it.block];
-    const int n = bd.n, lane = threadIdx.x & 31;
-    const int64_t eidx = (int64_t)it.q0 + (threadIdx.x >> 5);
-    if (eidx >= (int64_t)n * n) return;  // uniform per warp
-    const int q = (int)(eidx / n), r = (int)(eidx % n);
+    const int n = bd.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q = it.q0 & 0xffff, r0 = (it.q0 >> 16) * kDenseCols + warp;
     const int64_t tbase = (int64_t)bd.op * nslots;
     const double *nv = ninv + (int64_t)bd.op * npix;
-    double acc = 0.0;
-    for (int e = 0; e < bd.npairs; ++e) {
-        const PairEntry pe = entries[bd.pair0 + e];
-        const int64_t P = pe.P, Q = pe.Q, m = pe.mmax;
-        const int64_t half = P * pe.nrho;  // P Q g
-        const int64_t T2 = 2 * half;
-        const double *trow = tb + tbase + pe.tab;
-        // the pixels coupled to q: the whole ring when the support covers it,
-        // else the arc |z_q| <= mmax (each pixel once)
-        const bool full = m >= half;
-        const int64_t Zq = (2 * (int64_t)q + 1) * Q;
-        int64_t lo = 0, hi = pe.nrho - 1;
-        if (!full) {  // ceil((Z - m - P) / 2P) .. floor((Z + m - P) / 2P)
-            const int64_t a = Zq - m - P, b = Zq + m - P, d2 = 2 * P;
-            lo = a >= 0 ? (a + d2 - 1) / d2 : -((-a) / d2);
-            hi = b >= 0 ? b / d2 : -((-b + d2 - 1) / d2);
-        }
-        // z of q and of r against pixel pm, reduced to (-half, half]; the
-        // lane's next pixel is 32 on (mod nrho), so both z move by a fixed
-        // step reduced once
-        const int64_t nr = pe.nrho;
-        int64_t pm = (lo + lane) % nr;
-        if (pm < 0) pm += nr;
-        const int64_t s32 = 32 % nr, dz = 2 * P * s32;
-        int64_t zq = wrap_half(Zq - (2 * pm + 1) * P, half, T2);
-        int64_t zr = wrap_half((2 * (int64_t)r + 1) * Q - (2 * pm + 1) * P, half, T2);
-        for (int64_t pp = lo + lane; pp <= hi; pp += 32) {
-            if (zq <= m && -zq <= m && zr <= m && -zr <= m) {
-                const double bq = trow[((zq < 0 ? -zq : zq) - pe.par) >> 1];
-                const double br = trow[((zr < 0 ? -zr : zr) - pe.par) >> 1];
-                acc = fma(bq * nv[pe.noff + pm * pe.nstride], br, acc);
-            }
-            pm += s32;
-            if (pm >= nr) pm -= nr;
-            zq -= dz;
-            if (zq <= -half) zq += T2;
-            zr -= dz;
-            if (zr <= -half) zr += T2;
-        }
-    }
+    double acc[NR];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) {
-        int k = q > r ? q - r : r - q;
-        if (n - k < k) k = n - k;
-        if (k < bd.dK) acc += td[tbase + bd.dtab + k];
-        out[(dense_storage ? bd.off_dense : bd.off_pband) + (int64_t)q * n + r] = acc;
-    }
-}
-
-// Large dense-format blocks: one thread per element (q, r), 256 elements of
-// a row-major block per CTA, every pixel of every coupled ring tested (the
-// warp's 32 elements share their row q, so the q test is uniform), the
-// separation index reduced to |dphi| <= pi.  FP64.
-__global__ void __launch_bounds__(256) k_sample_dense_rows(const SampleItem *__restrict__ items,
-                                                      const BlockDesc *__restrict__ blocks,
-                                                      const PairEntry *__restrict__ entries, int64_t nslots,
-                                                      int64_t npix, const double *__restrict__ tb,
-                                                      const double *__restrict__ td, const double *__restrict__ ninv,
-                                                      double *__restrict__ out, int dense_storage) {
-    const SampleItem it = items[blockIdx.x];
-    const BlockDesc bd = blocks[it.block];
-    const int n = bd.n;
-    const int64_t eidx = (int64_t)it.q0 + threadIdx.x;
-    if (eidx >= (int64_t)n * n) return;
-    const int q = (int)(eidx / n), r = (int)(eidx % n);
-    const int64_t tbase = (int64_t)bd.op * nslots;
-    const double *nv = ninv + (int64_t)bd.op * npix;
-    double acc = 0.0;
-    for (int e = 0; e < bd.npairs; ++e) {
-        const PairEntry pe = entries[bd.pair0 + e];
-        const int64_t P = pe.P, Q = pe.Q, m = pe.mmax;
-        const int64_t half = P * pe.nrho;  // P Q g
-        const int64_t T2 = 2 * half;
-        const double *trow = tb + tbase + pe.tab;
-        // z of q and of r against pixel p, reduced to (-half, half], moved
-        // by -2P per pixel
-        int64_t zq = wrap_half((2 * (int64_t)q + 1) * Q - P, half, T2);
-        int64_t zr = wrap_half((2 * (int64_t)r + 1) * Q - P, half, T2);
-        for (int p = 0; p < pe.nrho; ++p) {
-            if (zq <= m && -zq <= m && zr <= m && -zr <= m) {
-                const double bq = trow[((zq < 0 ? -zq : zq) - pe.par) >> 1];
-                const double br = trow[((zr < 0 ? -zr : zr) - pe.par) >> 1];
-                acc = fma(bq * nv[pe.noff + (int64_t)p * pe.nstride], br, acc);
+    for (int k = 0; k < NR; ++k) acc[k] = 0.0;
+    for (int e0 = 0; e0 < bd.npairs; e0 += kDenseWarps) {
+        for (int c0 = 0;; c0 += kDensePix) {
+            __syncthreads();  // the weights before are used
+            int left = 0;     // pixels of this warp's ring from c0 on
+            if (e0 + warp < bd.npairs) {
+                const PairEntry pe = entries[bd.pair0 + e0 + warp];
+                const int P = pe.P, m = pe.mmax, nr = pe.nrho, half = P * nr, T2 = 2 * half, d2 = 2 * P;
+                const int Zq = (2 * q + 1) * pe.Q;
+                int lo = 0, hi = nr - 1;
+                if (m < half) {  // ceil((Z - m - P) / 2P) .. floor((Z + m - P) / 2P)
+                    const int a = Zq - m - P, b = Zq + m - P;
+                    lo = a >= 0 ? (a + d2 - 1) / d2 : -((-a) / d2);
+                    hi = b >= 0 ? b / d2 : -((-b + d2 - 1) / d2);
+                }
+                const int len = hi - lo + 1;
+                int pm0 = lo % nr;
+                if (pm0 < 0) pm0 += nr;
+                left = len - c0;
+                if (lane == 0) {
+                    s_len[warp] = left;
+                    s_pm[warp] = pm0;
+                }
+                for (int i = lane; i < min(left, kDensePix); i += 32) {
+                    const int pm = (pm0 + c0 + i) % nr;
+                    const int z = wrap_half(Zq - (2 * pm + 1) * P, half, T2), az = z < 0 ? -z : z;
+                    wgt[warp][i] = az <= m ? tb[tbase + pe.tab + ((az - pe.par) >> 1)] *
+                                                 nv[pe.noff + (int64_t)pm * pe.nstride]
+                                           : 0.0;
+                }
+            } else if (lane == 0) {
+                s_len[warp] = 0;
             }
-            zq -= 2 * P;
-            if (zq <= -half) zq += T2;
-            zr -= 2 * P;
-            if (zr <= -half) zr += T2;
+            const int more = __syncthreads_or(left > kDensePix);
+            for (int k = 0; k < kDenseWarps; ++k) {
+                const int len = min(s_len[k], kDensePix);
+                if (len <= 0) continue;
+                const PairEntry pe = entries[bd.pair0 + e0 + k];
+                const int P = pe.P, m = pe.mmax, nr = pe.nrho, half = P * nr, T2 = 2 * half;
+                const double *T = tb + tbase + pe.tab;
+                // the lane's next pixel is 32 on (mod nr): z moves by a step reduced once
+                const int dz = 2 * P * (32 % nr), pm = (s_pm[k] + c0 + lane) % nr;
+#pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    const int r = r0 + kDenseWarps * u;
+                    if (r > q) break;  // uniform in the warp
+                    int z = wrap_half((2 * r + 1) * pe.Q - (2 * pm + 1) * P, half, T2);
+                    double v = acc[u];
+                    for (int i = lane; i < len; i += 32) {
+                        const int az = z < 0 ? -z : z;
+                        if (az <= m) v = fma(wgt[k][i], T[(az - pe.par) >> 1], v);
+                        z -= dz;
+                        if (z <= -half) z += T2;
+                    }
+                    acc[u] = v;
+                }
+            }
+            if (!more) break;
         }
     }
-    int k = q > r ? q - r : r - q;
-    if (n - k < k) k = n - k;
-    if (k < bd.dK) acc += td[tbase + bd.dtab + k];
-    out[(dense_storage ? bd.off_dense : bd.off_pband) + (int64_t)q * n + r] = acc;
+    double *M = out + (dense_storage ? bd.off_dense : bd.off_pband);
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+        const int r = r0 + kDenseWarps * u;
+        if (r > q) break;
+        double v = acc[u];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0) {
+            int k = q - r;
+            if (n - k < k) k = n - k;
+            if (k < bd.dK) v += td[tbase + bd.dtab + k];
+            M[(int64_t)q * n + r] = v;
+            M[(int64_t)r * n + q] = v;
+        }
+    }
 }
 
 }  // namespace sympix
@@ -199,12 +194,8 @@ extern "C" int sympix_sample_blocks(sympix_plan_t pl, const double *ninv, int pr
     }
     trace_mark(pl, st, "k_sample_pband");
     if (!pl->items_dense.empty())
-        k_sample_dense<<<(unsigned)pl->items_dense.size(), 32 * kDenseItemElems, 0, st>>>(
+        k_sample_dense<<<(unsigned)pl->items_dense.size(), 32 * kDenseWarps, 0, st>>>(
             pl->d_items_dense.p, pl->d_blocks.p, pl->d_entries.p, pl->nslots, pl->grid->npix, pl->d_tab_b.p,
-            pl->d_tab_d.p, ninv, blocks, dense ? 1 : 0);
-    if (!pl->items_dense_rows.empty())
-        k_sample_dense_rows<<<(unsigned)pl->items_dense_rows.size(), 256, 0, st>>>(
-            pl->d_items_dense_rows.p, pl->d_blocks.p, pl->d_entries.p, pl->nslots, pl->grid->npix, pl->d_tab_b.p,
             pl->d_tab_d.p, ninv, blocks, dense ? 1 : 0);
     trace_mark(pl, st, "k_sample_dense");
     cudaError_t e = cudaGetLastError();
