@@ -366,6 +366,9 @@ struct sympix_plan_s {
     sympix::DevBuf<float> d_tab_blo;         // [op][nslots] FP32 remainder b - hi
     sympix::DevBuf<float> d_tab_d32, d_tab_dlo; // the same split of d
     sympix::DevBuf<float> d_ninv32, d_ninvlo;   // [op][npix] split of N^-1, per sampling call
+    // several operators: the kernel table's order of the slots, how many
+    // operators reach each slot, and the operators by radius (largest first)
+    sympix::DevBuf<int32_t> d_slot_perm, d_slot_need, d_op_order;
     sympix::DevBuf<double> d_rec;            // recurrence coefficients
     sympix::DevBuf<BlockDesc> d_blocks;
     sympix::DevBuf<PairEntry> d_entries;

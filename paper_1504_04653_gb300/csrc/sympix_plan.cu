@@ -290,6 +290,31 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
     k_support_slots<<<(npairs + 127) / 128, 128>>>(npairs, pl->d_pairs.p, grid->d_theta.p, pl->d_slot_u.p,
                                                    pl->d_slot_pair.p);
 
+    if (nops > 1) {
+        std::vector<int32_t> by_radius(nops), need((size_t)nslots), perm((size_t)nslots);
+        std::iota(by_radius.begin(), by_radius.end(), 0);
+        if (!tiles)
+            std::stable_sort(by_radius.begin(), by_radius.end(),
+                             [&](int x, int y) { return pl->r_s[x] > pl->r_s[y]; });
+        int64_t same = 0;  // slots of same-ring pairs (the first ones)
+        for (int pi = 0; pi < npairs; ++pi) {
+            const CanonPair &cp = pl->pairs[pi];
+            const int par = (cp.na / cp.g + cp.nb / cp.g) & 1;
+            int reach = nops;  // operators whose coupled classes include the level, largest radius first
+            for (int k = 0; k < cp.kmax; ++k) {
+                while (reach > 0 && pl->pair_mmax[(size_t)pi * nops + by_radius[reach - 1]] < par + 2 * k) --reach;
+                need[(size_t)(cp.slot0 + k)] = reach;
+            }
+            if (cp.a == cp.b) same += cp.kmax;
+        }
+        std::iota(perm.begin(), perm.end(), 0);
+        auto more = [&](int x, int y) { return need[x] > need[y]; };
+        std::stable_sort(perm.begin(), perm.begin() + same, more);
+        std::stable_sort(perm.begin() + same, perm.end(), more);
+        if ((rc = pl->d_slot_need.upload(need)) || (rc = pl->d_slot_perm.upload(perm)) ||
+            (rc = pl->d_op_order.upload(by_radius)))
+            return fail(rc);
+    }
     // blocks and their coupled neighbour rings (DP grids: one block per band)
     if (tiles && (rc = plan_tile_blocks(pl, index, ring0 / kk, ring1 / kk))) return fail(rc);
     const int nb = ring1 - ring0;

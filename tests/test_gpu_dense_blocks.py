@@ -38,3 +38,27 @@ def test_dense_sampling_matches_oracle(lmax, radii, storage):
             assert np.max(np.abs(M - ref)) <= 1e-10 * np.max(np.abs(ref)), (o, j, n)
             sizes.add((n + 63) // 64)
     assert {1, 2} <= sizes
+
+
+def test_table_of_several_radii():
+    """The kernel values of several operators with their own radii equal those
+    of plans with one operator, bit for bit, wherever they are coupled."""
+    import torch
+    from paper_1504_04653_gb300 import sympix as S
+    lmax, radii = 60, [0.1, 0.45, 0.02, 0.3, 0.3, 0.07, 0.6, 0.15, 0.25, 0.01, 0.5]
+    grid = S.Grid(lmax)
+    bl = np.stack([W.gaussian_beam(lmax, 60.0 + 30 * o) for o in range(len(radii))])
+    dl = np.stack([W.prior(lmax) * (1 + o) for o in range(len(radii))])
+    many = S.Plan(grid, radii)
+    S.sympix_kernel_table(many, torch.tensor(bl).cuda(), torch.tensor(dl).cuda())
+    for o, r in enumerate(radii):
+        one = S.Plan(grid, [r])
+        S.sympix_kernel_table(one, torch.tensor(bl[o:o + 1]).cuda(), torch.tensor(dl[o:o + 1]).cuda())
+        for j in (0, 7, 30, 44):
+            m = one.support(0, j, 12)
+            for rho in range(max(0, j - 12), min(grid.nrings, j + 13)):
+                if m[rho - j + 12] < 0:
+                    continue
+                count = int(m[rho - j + 12]) // 2 + 1
+                for a, b in zip(many.table(o, j, rho, count), one.table(0, j, rho, count)):
+                    assert a is None and b is None or np.array_equal(a, b), (o, j, rho)
