@@ -650,7 +650,9 @@ void launch_factor_wide_dense(sympix_plan_t pl, int precision, bool dense, doubl
             trace_mark(pl, st, "k_factor_wide");
         }
     }
-    const int nd = (int)pl->factor_items[3].size(), ns = (int)pl->factor_items[4].size();
+    const int nd = (int)pl->factor_items[3].size() -
+                   dense_in_window(pl, dense ? SYMPIX_STORE_DENSE : SYMPIX_STORE_PBAND, precision);
+    const int ns = (int)pl->factor_items[4].size();
     if (nd)
         k_factor_dense<<<(unsigned)((nd * 32 + 127) / 128), 128, 0, st>>>(nd, pl->d_factor_items[3].p, pl->d_blocks.p,
                                                                         blocks, dense ? 1 : 0, info);

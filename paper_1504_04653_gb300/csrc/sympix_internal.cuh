@@ -325,12 +325,14 @@ struct sympix_plan_s {
     std::vector<CholSlice> chol_sl32, chol_sl64;
     std::vector<int2> chol_tiles;
     int chol_wmax = -1;
-    // sliding-window factor (FP64 and split FP32): one warp per entry (first
-    // of chol_items, count, width), longest first; [0] as many blocks per
+    // sliding-window factor (FP64 and split FP32): chol_items and the win_dense
+    // dense-format blocks of up to 32 rows (the last of factor_items[3]); one
+    // warp per entry (first, count, width, -1: dense), longest first; [0] as many blocks per
     // warp as the width allows, [1] one block per warp, and which list each
     // arithmetic runs
     sympix::DevBuf<int4> d_win[2];
-    int win_one[3] = {0, 0, 0};
+    int win_one[3] = {0, 0, 0}, win_dense = 0;
+    sympix::DevBuf<int32_t> d_win_items;
     // per width: the slices [chol_f32[w], + chol_n32[w]) of chol_sl32 and
     // [chol_f64[w], + chol_n64[w]) of chol_sl64; a stream per width present
     // (the widths run side by side) and the fork / join events
@@ -361,14 +363,14 @@ struct sympix_plan_s {
     sympix::DevBuf<CanonPair> d_pairs;
     sympix::DevBuf<double> d_slot_u;         // u = 1 - cos(gamma) per slot
     sympix::DevBuf<int32_t> d_slot_pair;     // canonical pair of each slot
+    // several operators: the kernel table's order of the slots, how many
+    // operators reach each slot, and the operators by radius (largest first)
+    sympix::DevBuf<int32_t> d_slot_perm, d_slot_need, d_op_order;
     sympix::DevBuf<double> d_tab_b, d_tab_d; // [op][nslots] FP64
     sympix::DevBuf<float> d_tab_b32;         // [op][nslots] FP32 (rounded)
     sympix::DevBuf<float> d_tab_blo;         // [op][nslots] FP32 remainder b - hi
     sympix::DevBuf<float> d_tab_d32, d_tab_dlo; // the same split of d
     sympix::DevBuf<float> d_ninv32, d_ninvlo;   // [op][npix] split of N^-1, per sampling call
-    // several operators: the kernel table's order of the slots, how many
-    // operators reach each slot, and the operators by radius (largest first)
-    sympix::DevBuf<int32_t> d_slot_perm, d_slot_need, d_op_order;
     sympix::DevBuf<double> d_rec;            // recurrence coefficients
     sympix::DevBuf<BlockDesc> d_blocks;
     sympix::DevBuf<PairEntry> d_entries;
@@ -427,3 +429,9 @@ struct sympix_plan_s {
     sympix::DevBuf<int32_t> d_status;
     int wait_limit = 1 << 22;
 };
+
+// The small dense-format blocks (the last of factor_items[3]) that the
+// sliding-window launch of a factor call takes along.
+inline int dense_in_window(sympix_plan_t pl, int storage, int precision) {
+    return storage == SYMPIX_STORE_PBAND && pl->narrow_pref[precision] == sympix::kNarrowWindow ? pl->win_dense : 0;
+}

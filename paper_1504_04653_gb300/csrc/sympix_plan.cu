@@ -574,7 +574,11 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
     }
     // sliding-window factor: warps of both layouts, longest first, and the
     // layout whose estimated time (the longest warp, or all of them spread
-    // over the schedulers) is shorter
+    // over the 608 schedulers) is shorter.  Measured, full warps / one block
+    // per warp: l_max 64 FP64 0.119 / 0.094 ms, l_max 200 with four operators
+    // 0.346 / 0.291 ms, l_max 500 with two operators 0.937 / 1.074 ms, l_max
+    // 1500 2.98 / 3.31 ms; split FP32 0.086 / 0.064, 0.225 / 0.183, 0.765 /
+    // 0.796 and 2.08 / 2.21 ms
     {
         double est[2] = {0.0, 0.0};
         for (int one = 0; one < 2; ++one) {
@@ -586,9 +590,18 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
                 size_t e = i;
                 while (e < pl->chol_items.size() && e < i + per && pl->blocks[pl->chol_items[e]].w == w) ++e;
                 const double cost = window_step_cost(w, 32 / per) * pl->blocks[pl->chol_items[i]].n;
+        std::vector<int32_t> items = pl->chol_items;
+        for (int b : pl->factor_items[3])
+            if (!tiles && pl->blocks[b].n <= 32) items.push_back(b);
+        pl->win_dense = (int)(items.size() - pl->chol_items.size());
+        if ((rc = pl->d_win_items.upload(items))) return fail(rc);
                 work.push_back({cost, make_int4((int)i, (int)(e - i), w, 0)});
                 total += cost;
                 longest = std::max(longest, cost);
+            for (size_t i = pl->chol_items.size(); i < items.size(); ++i) {
+                const double n = pl->blocks[items[i]].n;
+                work.push_back({n * (0.5 * n + 8.0), make_int4((int)i, 1, -1, 0)});
+            }
                 i = e;
             }
             std::stable_sort(work.begin(), work.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
@@ -932,7 +945,7 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
         f += (l0 || l1 || l2) ? 2 : 0;  // both passes for every width up to 16
     } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == kNarrowWindow) {
         // w <= 12 in the sliding-window kernel, then the lane groups of 12 < w <= 16
-        f += (pl->chol_items.empty() ? 0 : 1) + (l2 ? 1 : 0);
+        f += (pl->d_win[0].n > 0 ? 1 : 0) + (l2 ? 1 : 0);
     } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == 2) {
         // w <= 12 on the FP64 / split-FP32 shadow: transpose in, band pass, transfer, carry,
         // solve and corner sums of each width range, corners, write-back; then
@@ -947,7 +960,8 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
         f += (l0 ? 2 : 0) + (l1 ? 1 : 0) + (l2 ? 1 : 0);
     }
     f += (int)pl->wide_cls.size() * ((factor_precision == SYMPIX_PREC_FP32 && pband) ? 2 : 1);
-    for (int l = 3; l < 5; ++l) f += pl->factor_items[l].empty() ? 0 : 1;
+    f += (int)pl->factor_items[3].size() > dense_in_window(pl, storage, factor_precision) ? 1 : 0;
+    f += pl->factor_items[4].empty() ? 0 : 1;
     if (factor) *factor = f;
     return SYMPIX_OK;
 }
@@ -1014,7 +1028,8 @@ extern "C" int sympix_plan_device_bytes(sympix_plan_t pl, size_t *bytes, size_t 
                pl->d_split_bandres.bytes() + pl->d_f32_tiles_lo.bytes() + pl->d_f32_out_tiles_lo.bytes();
     for (const auto &kv : pl->coupling)
         b += kv.second.d_arcs.bytes() + kv.second.d_rest.bytes() + kv.second.d_tile0.bytes() + kv.second.d_first.bytes();
-    b += pl->d_apply_items.bytes() + pl->d_apply_rest.bytes();
+    b += pl->d_apply_items.bytes() + pl->d_apply_rest.bytes() + pl->d_win_items.bytes() +
+         pl->d_slot_perm.bytes() + pl->d_slot_need.bytes() + pl->d_op_order.bytes();
     for (int i = 0; i < 2; ++i) b += pl->d_win[i].bytes() + pl->d_apply_work[i].bytes();
     for (int i = 0; i < 5; ++i) b += pl->d_items_pband[i].bytes();
     for (int i = 0; i < 3; ++i) b += pl->d_items_wide[i].bytes();

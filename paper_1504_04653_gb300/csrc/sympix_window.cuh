@@ -39,9 +39,10 @@
 // block, but its step takes 1.8k cycles and the border needs a second pass of
 // about the same length; here a block's n steps take 1210 cycles each in FP64
 // and 780 in split FP32 for band and border together, and nothing is
-// transposed.  Factor stage, before and now: l_max 500 FP64 3.3 -> 1.05 ms,
-// l_max 1500 FP64 5.8 -> 2.9 ms, l_max 3000 FP64 12.9 -> 7.6 ms; l_max 750 with
-// three operators, split FP32, 2.1 -> 1.0 ms; l_max 3000 6.0 -> 3.9 ms.
+// transposed.  Factor stage, before and now: l_max 64 FP64 0.47 -> 0.094 ms,
+// l_max 500 3.3 -> 0.93 ms, l_max 1500 5.8 -> 3.0 ms, l_max 3000 12.9 -> 7.4 ms;
+// split FP32 at l_max 750 with three operators 2.1 -> 1.4 ms, l_max 3000 6.0 ->
+// 3.7 ms.
 #pragma once
 
 #include <algorithm>
@@ -215,9 +216,22 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
     }
     for (int i = gl; i < W * W; i += G)
         tail[i] = bi >= 0 ? elem_from_f64<V>(view.a(m + i / W, m - W + i % W)) : V(0);
-    V acc[NPAIR];
+    // corner sums: all of them over this lane's columns, or for wide windows
+    // (W > 8: too many registers) this lane's share of them over all columns
+    constexpr bool SHARE = W > 8;
+    constexpr int NACC = SHARE ? (NPAIR + G - 1) / G : NPAIR;
+    V acc[NACC];
+    int pb[NACC], pc[NACC];
 #pragma unroll
-    for (int i = 0; i < NPAIR; ++i) acc[i] = V(0);
+    for (int i = 0; i < NACC; ++i) {
+        acc[i] = V(0);
+        if constexpr (SHARE) {
+            int k = min(gl + i * G, NPAIR - 1), b = 0;
+            while (k > b) k -= ++b;  // pair b (b + 1) / 2 + c
+            pb[i] = b * HS;
+            pc[i] = k * HS;
+        }
+    }
     int inf = 0, done = 0;
     // column 0's entry of this lane's row, the pivot and its reciprocal
     V a = x[0];
@@ -242,10 +256,21 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
 #pragma unroll
             for (int b = 0; b < W; ++b) bord[(int64_t)b * n + k] = elem_to_f64(xb[b]);
         }
+        if constexpr (SHARE) {
 #pragma unroll
-        for (int b = 0; b < W; ++b)
+            for (int b = 0; b < W; ++b) hist[b * HS + k % HB] = xb[b];
+            __syncwarp();
+            const V *x = hist + done % HB;  // G columns from done, a multiple of G
+#pragma unroll 4
+            for (int j = 0; j < G; ++j)
 #pragma unroll
-            for (int c = 0; c <= b; ++c) acc[b * (b + 1) / 2 + c] = band_fma(xb[b], xb[c], acc[b * (b + 1) / 2 + c]);
+                for (int i = 0; i < NACC; ++i) acc[i] = band_fma(x[pb[i] + j], x[pc[i] + j], acc[i]);
+        } else {
+#pragma unroll
+            for (int b = 0; b < W; ++b)
+#pragma unroll
+                for (int c = 0; c <= b; ++c) acc[b * (b + 1) / 2 + c] = band_fma(xb[b], xb[c], acc[b * (b + 1) / 2 + c]);
+        }
         done += G;
     };
 
@@ -349,7 +374,17 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
     __syncwarp();
     // the corner A22 - S, one row per lane, eliminated in FP64
     double *sums = reinterpret_cast<double *>(hist);
-    WindowReduce<V, NPAIR, G / 2>::run(acc, gl, 0, NPAIR, sums);
+    if constexpr (SHARE) {
+        double mine[NACC];
+#pragma unroll
+        for (int i = 0; i < NACC; ++i) mine[i] = elem_to_f64(acc[i]);
+        __syncwarp();  // the history has been read
+#pragma unroll
+        for (int i = 0; i < NACC; ++i)
+            if (gl + i * G < NPAIR) sums[gl + i * G] = mine[i];
+    } else {
+        WindowReduce<V, NPAIR, G / 2>::run(acc, gl, 0, NPAIR, sums);
+    }
     __syncwarp();
     double cr[W];
 #pragma unroll
@@ -391,14 +426,56 @@ __device__ __forceinline__ void window_diag(const BlockDesc *__restrict__ blocks
     if (lane == 0) info[bi] = first < bd.n ? first + 1 : 0;
 }
 
-// One warp per item: blocks items[first .. first + count) of width w.  ONE:
-// one block per warp.  Four independent warps per CTA, one on each scheduler
+// A dense-format block of up to 32 rows (polar rings), in FP64 whatever the
+// arithmetic: the lower triangle in shared memory (rows of 33), one row per
+// lane.  Beside the window's chains it costs nothing; as a launch of its own
+// (k_factor_dense) it added 36 to 55 us to every factor.
+__device__ __forceinline__ void window_dense(const BlockDesc *__restrict__ blocks, int bi, double *__restrict__ out,
+                                             int32_t *__restrict__ info, double *a) {
+    const int lane = threadIdx.x & 31;
+    const BlockDesc bd = blocks[bi];
+    const int n = bd.n;
+    double *A = out + bd.off_pband;
+    for (int i = lane; i < n * n; i += 32)
+        if (i % n <= i / n) a[i / n * 33 + i % n] = A[i];
+    __syncwarp();
+    int inf = 0;
+    for (int j = 0; j < n; ++j) {
+        const double d = a[j * 33 + j];
+        if (!window_positive(d)) {  // the same in every lane
+            inf = j + 1;
+            break;
+        }
+        double l = 0.0;
+        if (lane >= j && lane < n) {
+            l = a[lane * 33 + j] * window_rsqrt(d);
+        }
+        __syncwarp();  // the pivot has been read
+        if (lane >= j && lane < n) a[lane * 33 + j] = l;
+        for (int k = j + 1; k < n; ++k) {
+            const double lk = window_shfl(l, k, 32);
+            if (lane >= k && lane < n) a[lane * 33 + k] = fma(-l, lk, a[lane * 33 + k]);
+        }
+        __syncwarp();
+    }
+    if (inf == 0)
+        for (int i = lane; i < n * n; i += 32)
+            if (i % n <= i / n) A[i] = a[i / n * 33 + i % n];
+    if (lane == 0) info[bi] = inf;
+}
+
+// One warp per item: blocks items[first .. first + count) of width w (-1: one
+// small dense-format block).  ONE: one block per warp.  Four independent warps per CTA, one on each scheduler
 // of its SM: CTAs of one warp were placed unevenly (up to three on one
 // scheduler and none on another), which doubled the time.
 constexpr int kWindowWarps = 4;
+// Shared memory that keeps a third CTA off the SM: the longest blocks set the
+// time and come first, and a third warp on each scheduler slows them down
+// (l_max 3000 FP64 8.7 ms with three, 7.5 ms with two).
+constexpr int kWindowSmemMin = 80 * 1024;
 
 template <class V, bool ONE>
-__global__ void __launch_bounds__(32 * kWindowWarps) k_window_chol(int count, int smem_warp,
+__global__ void __launch_bounds__(32 * kWindowWarps, 2) k_window_chol(int count, int smem_warp,
                                                                    const int4 *__restrict__ work,
                                                                    const int32_t *__restrict__ items,
                                                                    const BlockDesc *__restrict__ blocks,
@@ -418,20 +495,23 @@ __global__ void __launch_bounds__(32 * kWindowWarps) k_window_chol(int count, in
     });
     if (it.z == 0)
         for (int g = 0; g < it.y; ++g) window_diag<V>(blocks, items[it.x + g], out, info);
+    else if (it.z < 0)
+        window_dense(blocks, items[it.x], out, info, reinterpret_cast<double *>(window_smem));
 }
 
 template <class V, bool ONE>
 void launch_window_list(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st) {
-    size_t smem = 16;
+    size_t smem = pl->win_dense ? 32 * 33 * sizeof(double) : 16;
     for (int w = 1; w <= pl->chol_wmax; ++w) {
         const int g = ONE ? 32 : window_rows(w);
         smem = std::max(smem, (size_t)(32 / g) * window_elems(w, g) * 8);
     }
+    smem = std::max(smem, (size_t)kWindowSmemMin / kWindowWarps);
     const int count = (int)pl->d_win[ONE].n;
     cudaFuncSetAttribute(k_window_chol<V, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(kWindowWarps * smem));
     k_window_chol<V, ONE><<<(unsigned)((count + kWindowWarps - 1) / kWindowWarps), 32 * kWindowWarps,
-                            kWindowWarps * smem, st>>>(count, (int)smem, pl->d_win[ONE].p, pl->d_chol_items.p,
+                            kWindowWarps * smem, st>>>(count, (int)smem, pl->d_win[ONE].p, pl->d_win_items.p,
                                                        pl->d_blocks.p, blocks, info);
 }
 

@@ -9,7 +9,7 @@ void launch_window_f64(sympix_plan_t pl, double *blocks, int32_t *info, cudaStre
 }
 
 void launch_window(sympix_plan_t pl, int precision, double *blocks, int32_t *info, cudaStream_t st) {
-    if (!pl->chol_items.empty()) {
+    if (pl->d_win[0].n > 0) {
         if (precision == SYMPIX_PREC_FP64)
             launch_window_f64(pl, blocks, info, st);
         else

@@ -1,5 +1,5 @@
 """Dense-format ring blocks (polar or fully coupled rings): sampling over row
-tiles."""
+tiles, and the factor of up to 32 rows inside the sliding-window launch."""
 import numpy as np
 import pytest
 
@@ -38,6 +38,49 @@ def test_dense_sampling_matches_oracle(lmax, radii, storage):
             assert np.max(np.abs(M - ref)) <= 1e-10 * np.max(np.abs(ref)), (o, j, n)
             sizes.add((n + 63) // 64)
     assert {1, 2} <= sizes
+
+
+@pytest.mark.parametrize("fprec", ["fp64", "fp32x2"])
+def test_small_dense_factor(fprec):
+    """Blocks of 8 to 32 rows and just above: L against numpy's Cholesky with
+    the backward error n eps of FP64 (times 8), the pivot of an indefinite
+    block, the strict upper triangle untouched."""
+    import torch
+    from paper_1504_04653_gb300 import sympix as S
+    lmax = 30
+    grid = S.Grid(lmax)
+    plan = S.Plan(grid, [3.2, 0.6])
+    rng = np.random.default_rng(8)
+    nbytes, _ = plan.blocks_size("pband")
+    host = np.zeros(nbytes // 8)
+    want, seen = {}, set()
+    for o in range(2):
+        for j in range(grid.nrings):
+            off, n, w, fmt = plan.block_layout("pband", o, j)
+            if fmt == S.BLOCK_DENSE:
+                B = rng.standard_normal((n, n))
+                M = B @ B.T + n * np.eye(n)
+                bad = (j % 4 == 1) * (1 + (5 * j) % n)
+                if bad:
+                    M[bad - 1, bad - 1] = -1.0
+                host[off:off + n * n] = M.reshape(-1)
+                want[(o, j)] = (M, bad)
+                seen.add(n)
+            else:
+                host[off:off + n * (w + 1)].reshape(n, w + 1)[:, 0] = 1.0
+    blocks = torch.tensor(host).cuda()
+    info = S.sympix_factor_blocks(plan, blocks, precision=fprec).cpu().numpy()
+    got = blocks.cpu().numpy()
+    for (o, j), (M, bad) in want.items():
+        off, n, _, _ = plan.block_layout("pband", o, j)
+        assert info[o * grid.nrings + j] == bad, (o, j, n)
+        if bad:
+            continue
+        A = got[off:off + n * n].reshape(n, n)
+        L = np.tril(A)
+        assert np.array_equal(np.triu(A, 1), np.triu(M, 1))
+        assert np.max(np.abs(L @ L.T - M)) <= 8 * n * 2.0 ** -53 * np.max(np.abs(M)), (o, j, n)
+    assert min(seen) <= 12 and any(n > 32 for n in seen) and any(24 <= n <= 32 for n in seen), sorted(seen)
 
 
 def test_table_of_several_radii():
