@@ -405,7 +405,7 @@ int sympix_sample_coupling(sympix_plan_t plan, const double *ninv, int delta, do
  *   x, y          device FP64 [nops][npix] in pixel numbering (must not
  *                 alias); y is written at the planned rings' pixels.  A block
  *                 whose factorisation failed (info != 0) passes x through.
- * FP64, one warp per block.  Asynchronous. */
+ * FP64.  Asynchronous. */
 int sympix_apply(sympix_plan_t plan, int storage, const double *blocks, const int32_t *info, const double *x,
                  double *y, void *stream);
 

@@ -7,6 +7,10 @@
 //   L11 L11^T = A11,   L21 = A21 L11^-T,   L22 L22^T = A22 - L21 L21^T.
 //
 // Kernels, by band width and arithmetic (the plan sorts blocks into lists):
+//   w <= 12 (FP64, split FP32, periodic-band storage), the default: the
+//       sliding-window kernel, band, border and corner in one pass by the lanes
+//       of a warp (sympix_window.cuh), with the dense-format blocks of up to
+//       32 rows in the same launch.
 //   w <= 8 (FP64, split FP32) and w <= 16 (FP32 on pband storage):
 //       two passes.  The band pass runs one lane per block with the active
 //       (w+1) x (w+1) triangle in registers and band rows staged into
@@ -32,8 +36,8 @@
 // Files: sympix_factor_kernels.cuh (views, staging, the templated FP32
 // passes), sympix_factor_lanes.cu (FP64 / split FP32 band and border
 // kernels), sympix_factor_f32.cu and sympix_factor_fused.cu (the FP32
-// path), sympix_factor_wide.cu (wide bands, dense blocks), this file (the
-// entry point).
+// path), sympix_factor_wide.cu (wide bands, dense blocks), sympix_window*
+// (the sliding window), this file (the entry point).
 #include "sympix_chol.cuh"
 #include "sympix_factor_kernels.cuh"
 
