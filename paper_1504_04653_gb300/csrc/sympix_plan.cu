@@ -581,27 +581,27 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
     // 0.796 and 2.08 / 2.21 ms
     {
         double est[2] = {0.0, 0.0};
+        std::vector<int32_t> items = pl->chol_items;
+        for (int b : pl->factor_items[3])
+            if (!tiles && pl->blocks[b].n <= 32) items.push_back(b);
+        pl->win_dense = (int)(items.size() - pl->chol_items.size());
+        if ((rc = pl->d_win_items.upload(items))) return fail(rc);
         for (int one = 0; one < 2; ++one) {
             std::vector<std::pair<double, int4>> work;
             double total = 0.0, longest = 0.0;
+            for (size_t i = pl->chol_items.size(); i < items.size(); ++i) {
+                const double n = pl->blocks[items[i]].n;
+                work.push_back({n * (0.5 * n + 8.0), make_int4((int)i, 1, -1, 0)});
+            }
             for (size_t i = 0; i < pl->chol_items.size();) {
                 const int w = pl->blocks[pl->chol_items[i]].w;
                 const int per = one ? 1 : 32 / window_rows(w);
                 size_t e = i;
                 while (e < pl->chol_items.size() && e < i + per && pl->blocks[pl->chol_items[e]].w == w) ++e;
                 const double cost = window_step_cost(w, 32 / per) * pl->blocks[pl->chol_items[i]].n;
-        std::vector<int32_t> items = pl->chol_items;
-        for (int b : pl->factor_items[3])
-            if (!tiles && pl->blocks[b].n <= 32) items.push_back(b);
-        pl->win_dense = (int)(items.size() - pl->chol_items.size());
-        if ((rc = pl->d_win_items.upload(items))) return fail(rc);
                 work.push_back({cost, make_int4((int)i, (int)(e - i), w, 0)});
                 total += cost;
                 longest = std::max(longest, cost);
-            for (size_t i = pl->chol_items.size(); i < items.size(); ++i) {
-                const double n = pl->blocks[items[i]].n;
-                work.push_back({n * (0.5 * n + 8.0), make_int4((int)i, 1, -1, 0)});
-            }
                 i = e;
             }
             std::stable_sort(work.begin(), work.end(), [](const auto &a, const auto &b) { return a.first > b.first; });

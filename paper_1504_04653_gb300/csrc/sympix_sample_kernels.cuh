@@ -438,14 +438,18 @@ void launch_pband(sympix_plan_t pl, const double *ninv, double *blocks, cudaStre
             case 8: k_sample_pband<PREC, 8, DENSE_OUT><<<(unsigned)ni, 128, 0, st>>>(SPX_ARGS); break;
             case 16: k_sample_pband<PREC, 16, DENSE_OUT><<<(unsigned)ni, 128, 0, st>>>(SPX_ARGS); break;
             case 32:
-                cudaFuncSetAttribute(k_sample_pband<PREC, 32, DENSE_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)wcs);
-                k_sample_pband<PREC, 32, DENSE_OUT><<<(unsigned)ni, 128, wcs, st>>>(SPX_ARGS);
+                if constexpr (PREC != 1 || DENSE_OUT) {
+                    cudaFuncSetAttribute(k_sample_pband<PREC, 32, DENSE_OUT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wcs);
+                    k_sample_pband<PREC, 32, DENSE_OUT><<<(unsigned)ni, 128, wcs, st>>>(SPX_ARGS);
+                }
                 break;
             default:
-                cudaFuncSetAttribute(k_sample_pband<PREC, 64, DENSE_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)wcs);
-                k_sample_pband<PREC, 64, DENSE_OUT><<<(unsigned)ni, 128, wcs, st>>>(SPX_ARGS);
+                if constexpr (PREC != 1 || DENSE_OUT) {
+                    cudaFuncSetAttribute(k_sample_pband<PREC, 64, DENSE_OUT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wcs);
+                    k_sample_pband<PREC, 64, DENSE_OUT><<<(unsigned)ni, 128, wcs, st>>>(SPX_ARGS);
+                }
                 break;
         }
 #undef SPX_ARGS
