@@ -20,8 +20,8 @@
 // about 30: 206 cycles a step in multiply, shuffle and multiply-add, 340 to
 // 410 measured with everything else a step issues, for n steps each way.  One
 // lane's recurrence per block (k_apply below, before: all widths) took about
-// 2 W FP64 instructions a step.  l_max 500, two operators: 1.34 -> 0.39 ms;
-// l_max 3000: 22.6 -> 3.0 ms (3.4 GB at l_max 3000, 0.5 ms).  Scaling the
+// 2 W FP64 instructions a step.  l_max 500, two operators: 1.34 -> 0.40 ms;
+// l_max 3000: 22.6 -> 2.9 ms (3.4 GB at l_max 3000, 0.5 ms).  Scaling the
 // rows' coefficients by the reciprocals beforehand takes the multiplication
 // out of the chain, but costs as many instructions: 3.03 ms at l_max 3000.
 //
@@ -45,6 +45,12 @@ __device__ __forceinline__ bool apply_normal(double x) { return window_normal(x)
 __device__ __forceinline__ bool apply_nonzero(double x) { return ((__double2hiint(x) << 1) | __double2loint(x)) != 0; }
 __device__ __forceinline__ double apply_recip(double x) { return apply_normal(x) ? apply_recip_normal(x) : 1.0 / x; }
 
+// 16 bytes at dst, the first `bytes` of them from src, the others zero
+__device__ __forceinline__ void cp_async16_part(double *dst, const double *src, int bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ double apply_shfl(double x, int src, int width) {
     return __shfl_sync(0xffffffffu, x, src, width);
 }
@@ -56,6 +62,7 @@ struct ApplyVec {
     int64_t ps;
 };
 
+// n = 0: an idle group (`band` is then any 16-byte aligned address).
 template <int W, int G>
 __device__ __forceinline__ void apply_band(const double *__restrict__ band, int n, ApplyVec v, unsigned char *smem) {
     constexpr int RG = W <= 8 ? 8 : 16, H = G / RG, NB = (W + H - 1) / H;
@@ -64,10 +71,13 @@ __device__ __forceinline__ void apply_band(const double *__restrict__ band, int 
     const int rw = r < W ? r : 0;  // lanes past the band read row 0; their values reach no one
     double *ring = reinterpret_cast<double *>(smem) + (lane / G) * apply_elems(W);
     double *cs = ring + NP * PE;  // the corner, [row][column]
-    const int m = band ? n - W : 0;
+    const int m = n > 0 ? n - W : 0;
     const double *bord = band + (int64_t)n * RL;
-    const int bend = band ? n * RL : 0;
-    auto issue = [&](int per) {  // rows of period `per` into their place of the ring
+    // Rows of period `per` into their place of the ring.  Rows past the m of
+    // L11 are read, times zero, and L defines none of their entries: they are
+    // staged as zeros.
+    const int bend = m * RL;
+    auto issue = [&](int per) {
         const double *src = band + per * PE + 2 * gl;
         double *dst = ring + (per % NP) * PE + 2 * gl;
         if (per >= 0 && (per + 1) * PE <= bend) {
@@ -75,15 +85,16 @@ __device__ __forceinline__ void apply_band(const double *__restrict__ band, int 
             for (int i = 0; i < PE; i += 2 * G)
                 if (i + 2 * G <= PE || i + 2 * gl < PE) cp_async16(dst + i, src + i);
         } else if (per >= 0) {
-            for (int i = 0; i + 2 * gl < PE; i += 2 * G)
-                if (per * PE + i + 2 * gl < bend) cp_async16(dst + i, src + i);
+            for (int i = 0; i + 2 * gl < PE; i += 2 * G) {
+                const int left = bend - (per * PE + i + 2 * gl);
+                cp_async16_part(dst + i, left > 0 ? src + i : band, left < 0 ? 0 : left < 2 ? 8 * left : 16);
+            }
         }
         cp_async_commit();
     };
-    for (int i = gl; i < NP * PE; i += G) ring[i] = 0.0;  // places no copy reaches are read, times zero
     for (int i = gl; i < W * W; i += G) {
         const int b = i / W, c = i % W;
-        cs[i] = band && c <= b ? __ldg(bord + (int64_t)b * n + m + c) : 1.0;
+        cs[i] = m > 0 && c <= b ? __ldg(bord + (int64_t)b * n + m + c) : 1.0;
     }
     int mtop = m;
 #pragma unroll
@@ -102,6 +113,11 @@ __device__ __forceinline__ void apply_band(const double *__restrict__ band, int 
     auto border = [&](int k) {  // columns k + h NB .. of border row r
 #pragma unroll
         for (int j = 0; j < NB; ++j) bn[j] = k < m && h * NB + j < W ? __ldg(bp + k + j) : 0.0;
+        if (H == 1 && k + W > m) {  // a block's last period: see below
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                if (k + j >= m) bn[j] = 0.0;
+        }
     };
     __syncwarp();
 #pragma unroll
@@ -149,13 +165,24 @@ __device__ __forceinline__ void apply_band(const double *__restrict__ band, int 
         rr = apply_nonzero(dn) ? rn : 0.0;
 #pragma unroll
         for (int j = 0; j < NB; ++j) zl[j] = H == 1 ? zs[j < W ? j : 0] : apply_shfl(z, h * NB + j, G);
+        if (H == 1 && k0 + W > m) {
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                if (k0 + j >= m) zl[j] = 0.0;
+        }
         if (h == 0 && r < W && k0 + r < m) v.y[(k0 + r) * v.ps] = z;
         __syncwarp();
         issue(p + NP);
     }
     cp_async_wait<0>();
+    // A block's last period reaches past the m columns of L21: into the corner,
+    // whose entries past the diagonal no one has written, and to rows whose z is
+    // zero times what may be infinite.  Neither joins the dot product.  With one
+    // block per warp that period is the last of the loop (the same test in the
+    // loop: l_max 500 with two operators 0.403 ms against 0.397).
 #pragma unroll
-    for (int j = 0; j < NB; ++j) dot = fma(bc[j], zl[j], dot);
+    for (int j = 0; j < NB; ++j)
+        if ((np - 1) * W + h * NB + j < m) dot = fma(bc[j], zl[j], dot);
 #pragma unroll
     for (int o = RG; o < G; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     // corner: lane b < W holds border row b
@@ -202,8 +229,10 @@ __device__ __forceinline__ void apply_band(const double *__restrict__ band, int 
     };
     load_z(pt * W);
     s = enter();
+    if (pt * W + r >= m) s = 0.0;
     load_z((pt - 1) * W);
     double xe = enter();  // entering values of the period before
+    if ((pt - 1) * W + r >= m) xe = 0.0;
     load_z((pt - 2) * W);
     cp_async_wait<NP - 1>();
     __syncwarp();
@@ -234,6 +263,7 @@ __device__ __forceinline__ void apply_band(const double *__restrict__ band, int 
         xe = zn;
 #pragma unroll
         for (int o = RG; o < G; o <<= 1) xe += __shfl_xor_sync(0xffffffffu, xe, o);
+        if (H == 1 && k0 - 2 * W + r >= m) xe = 0.0;
         load_z(k0 - 3 * W);
         if (h == 0 && r < W && k0 + r < m) v.y[(k0 + r) * v.ps] = yv;
         __syncwarp();
@@ -292,18 +322,19 @@ __global__ void __launch_bounds__(32 * kApplyWarps) k_apply_band(int count, int 
         constexpr int W = decltype(Wc)::value, G = ONE ? 32 : apply_lanes(W);
         if (it.z != W) return;
         const int g = lane / G;
-        const double *band = nullptr;
+        const double *band = Lbuf;
         int n = 0;
         ApplyVec v{x, y, 1};
         if (g < it.y) {
             const int bi = items[it.x + g];
             const BlockDesc bd = blocks[bi];
             v = vec(bd);
-            n = bd.n;
-            if (info[bi] == 0)
+            if (info[bi] == 0) {
+                n = bd.n;
                 band = Lbuf + bd.off_pband;
-            else
-                copy(v, n, lane % G, G);
+            } else {
+                copy(v, bd.n, lane % G, G);
+            }
         }
         __syncwarp();
         apply_band<W, G>(band, n, v, smem);
@@ -472,9 +503,9 @@ static void launch_apply_band(sympix_plan_t pl, const double *blocks, const int3
 // warps of both layouts, longest first.  One block per warp while that is at
 // most two warps per scheduler (608 of them): a step then takes 340 cycles
 // against 410 in a full warp, which serves 32 / G blocks.  Measured, one block
-// per warp / full: l_max 500 0.334 / 0.407 ms, with two operators (1002
-// blocks) 0.394 / 0.438 ms, l_max 1500 (1501 blocks) 1.52 / 1.45 ms, l_max 500
-// with four operators 0.62 / 0.48 ms, l_max 3000 4.41 / 3.00 ms.
+// per warp / full: l_max 500 0.344 / 0.433 ms, with two operators (1002
+// blocks) 0.403 / 0.449 ms, l_max 1500 (1501 blocks) 1.54 / 1.42 ms, l_max 500
+// with four operators 0.63 / 0.46 ms, l_max 3000 4.41 / 2.89 ms.
 int plan_apply(sympix_plan_t pl, const std::vector<int32_t> &order) {
     std::vector<int32_t> items;
     std::vector<int32_t> rest;
