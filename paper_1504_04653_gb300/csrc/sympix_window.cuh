@@ -83,17 +83,33 @@ __device__ __forceinline__ double window_rsqrt_normal(double x) {
 }
 __device__ __forceinline__ double window_rsqrt(double x) { return window_normal(x) ? window_rsqrt_normal(x) : rsqrt(x); }
 __device__ __forceinline__ DF window_rsqrt(DF x) { return band_rsqrt(x); }
-__device__ __forceinline__ bool window_normal(DF) { return true; }
 // What a column's entries are multiplied by: 1/sqrt(pivot) in FP64; 1/pivot in
 // split FP32, by the series of the residual r = 1 - x y of the FP32 estimate.
 __device__ __forceinline__ double window_factor_normal(double x) { return window_rsqrt_normal(x); }
-__device__ __forceinline__ double window_factor(double x) { return rsqrt(x); }
 __device__ __forceinline__ DF window_factor_normal(DF x) {
     const float y = window_rcp32(x.hi);
     const DF r = df_fma(DF(-y), x, DF(1.0f));
     return to_df(f2_fast_two_sum(y, y * (fmaf(r.hi, r.hi, r.hi) + r.lo)));
 }
-__device__ __forceinline__ DF window_factor(DF x) { return window_factor_normal(x); }
+// Whether 2^-64 <= |x| < 2^64: 1/x then has both its words among FP32's normal
+// numbers (alone it is flushed to zero for x > 2^126 and loses its low word
+// from 2^104 on), and so have a column's entries times it.
+__device__ __forceinline__ bool window_common(DF x) { return ((__float_as_uint(x.hi) >> 23) & 0xffu) - 63u < 128u; }
+__device__ __forceinline__ DF window_scale(DF x, float g) { return DF(x.hi * g, x.lo * g); }
+// For any x > 0: g, a power of two with x g^2 in [1, 4), and 1 / (x g^2).  The
+// column's entries times g then stand for them in the step.
+__device__ __forceinline__ DF window_factor_far(DF x, float &g) {
+    const bool tiny = x.hi < 0x1p-100f;  // may be subnormal
+    if (tiny) x = window_scale(x, 0x1p+100f);
+    const int e = (int)((__float_as_uint(x.hi) >> 23) & 0xffu) - 127;
+    g = __uint_as_float((unsigned)(127 - (e >> 1)) << 23);
+    x = window_scale(window_scale(x, g), g);
+    if (tiny) g *= 0x1p+50f;
+    return window_factor_normal(x);
+}
+// (FP64's 1/sqrt needs neither)
+__device__ __forceinline__ double window_scale(double x, float) { return x; }
+__device__ __forceinline__ double window_factor_far(double x, float &) { return window_factor_normal(x); }
 
 // x > 0 on the integer ALU (an FP64 compare costs as much as a multiply-add)
 __device__ __forceinline__ bool window_positive(double x) {
@@ -237,11 +253,24 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
     V a = x[0];
     if constexpr (H > 1) a = window_shfl(a, r, G);
     V d = window_shfl(x[0], 0, G);
-    V f = window_normal(d) ? window_factor_normal(d) : window_factor(d);
+    V f = window_factor_normal(d);
+    if constexpr (!LDL)
+        if (!window_normal(d)) f = rsqrt(d);
     if (gl == 0) spare[0] = V(0);
     cp_async_wait<NP - 1>();
     __syncwarp();
     convert(0);
+    // Split FP32: a pivot is at most its row's diagonal entry, so the entries of
+    // the rows that a period eliminates, looked at while it enters, say whether
+    // one of its pivots can be too large (or the entry too small) for 1/pivot.
+    // Such a period runs a copy of the steps with scaled columns.  A test per
+    // pivot instead cost 12 to 27 % (l_max 750, three operators 1.81 ms; one a
+    // period 1.44; none 1.42).
+    bool far = false;
+    if constexpr (LDL) {
+        __syncwarp();
+        far = __any_sync(0xffffffffu, gl < W && gl < m && !window_common(ring[(gl < W ? gl : 0) * RL]));
+    }
     int mtop = m;
 #pragma unroll
     for (int o = G; o < 32; o <<= 1) mtop = max(mtop, __shfl_xor_sync(0xffffffffu, mtop, o));
@@ -275,7 +304,8 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
     };
 
     const int np = (mtop + W - 1) / W;
-    for (int p = 0; p < np; ++p) {
+    auto period = [&](int p, auto FARc) {
+        constexpr bool FAR = decltype(FARc)::value;
         cp_async_wait<NP - 2>();  // period p + 1 has landed
         __syncwarp();
         convert(p + 1);
@@ -301,12 +331,17 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
             }
         };
         enter(std::integral_constant<int, 0>{});
+        [[maybe_unused]] const V dn = nxt[(gl < W ? gl : 0) * RL];
+        [[maybe_unused]] float g = 1.0f;
+        if constexpr (FAR) f = window_factor_far(d, g);
         StaticFor<0, W>::run([&](auto Sc) {
             constexpr int s = decltype(Sc)::value, s1 = (s + 1) % W, js1 = s1 % WC;
             const int i = p * W + s;
             if (inf == 0 && i < m && !window_positive(d)) inf = i + 1;
             const V src = r == s ? na : a;
-            const V t = src * f, left = LDL ? src : t;
+            V col = src;
+            if constexpr (FAR) col = window_scale(src, g);
+            const V t = col * f, left = LDL ? col : t;
             V base[WC];
 #pragma unroll
             for (int j = 0; j < WC; ++j) {
@@ -321,23 +356,29 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
             d = window_shfl(x[js1], s1 / WC * RG + s1, G);
             a = x[js1];
             if constexpr (H > 1) a = window_shfl(a, s1 / WC * RG + r, G);
-            f = window_factor_normal(d);
+            if constexpr (FAR)
+                f = window_factor_far(d, g);
+            else
+                f = window_factor_normal(d);
 #pragma unroll
             for (int j = 0; j < WC; ++j)
                 if (j != js1) update(j);
-            if (__any_sync(0xffffffffu, !window_normal(d))) f = window_factor(d);
+            if constexpr (!LDL)
+                if (__any_sync(0xffffffffu, !window_normal(d))) f = rsqrt(d);
             // column i's entries: rows of this period and the next, the border's
             // history; the pivot in its row's diagonal position
             V *pw = (r > s ? cur : nxt) + r * RL + (r > s ? r - s : W - (s - r));
             if (r >= W) pw = hist + (r - W) * HS + i % HB;
             if (h > 0 || r >= 2 * W) pw = spare + 1;
-            *pw = left;
+            *pw = LDL ? src : t;
             if (r == s && h == 0) {
                 cur[s * RL] = a0;
                 if constexpr (!LDL) prs[i % HB] = f0;
             }
             __syncwarp();
         });
+        if constexpr (FAR) f = window_factor_normal(d);
+        if constexpr (LDL) far = __any_sync(0xffffffffu, gl < W && (p + 1) * W + gl < m && !window_common(dn));
         // rows p W .. p W + W - 1 of L
         const int rows = min(W, m - p * W);
         const bool ok = inf == 0;
@@ -368,6 +409,14 @@ __device__ __forceinline__ void window_chol(const BlockDesc *__restrict__ blocks
         if ((p + 1) * W - done >= G) flush_border(ok);
         __syncwarp();
         issue(p + NP);
+    };
+    if constexpr (LDL) {
+        for (int p = 0; p < np;) {
+            for (; p < np && !far; ++p) period(p, std::false_type{});
+            for (; p < np && far; ++p) period(p, std::true_type{});
+        }
+    } else {
+        for (int p = 0; p < np; ++p) period(p, std::false_type{});
     }
     cp_async_wait<0>();
     while (done < np * W) flush_border(inf == 0);  // columns past m are zero
