@@ -201,35 +201,9 @@ void launch_f32_slices(sympix_plan_t pl, double *blocks, int32_t *info, cudaStre
     const size_t nout = hi_only ? pl->f32_out_tiles_hi.size() : pl->f32_out_tiles.size();
     const int2 *tin = hi_only ? pl->d_f32_tiles_hi.p : pl->d_f32_tiles.p;
     const int2 *tout = hi_only ? pl->d_f32_out_tiles_hi.p : pl->d_f32_out_tiles.p;
-    // w <= 8: band and border passes in separate CTAs of one launch; 9 <= w <=
-    // 12 (a few slices, but the longest chains): band pass, then the chunked
-    // border kernels on the side stream at the same time (a second cooperative
-    // launch would wait for the first to finish).  While that path is still
-    // running, the main stream factors the dense-format blocks and writes the
-    // other slices back: l_max 3000 step 3.27 -> 3.23 ms (the two then share
-    // the memory; a transpose of its own at the start of the side stream made
-    // that path no shorter).
-    const bool side = !hi_only && f32_side_path(pl);
-    const int n8 = pl->f32_slices_w8;
-    auto write_back = [&](const int2 *tiles, size_t count) {
-        if (count)
-            k_f32_out<float><<<(unsigned)count, 256, 0, st>>>(tiles, sl, pl->d_f32_items.p, pl->d_blocks.p, info,
-                                                             pl->d_shadow_il.p, pl->d_l21_il.p, blocks);
-    };
     k_f32_shadow_in<float><<<(unsigned)nin, 256, 0, st>>>(tin, sl, pl->d_f32_items.p, pl->d_blocks.p, blocks,
                                                    pl->d_shadow_il.p);
     trace_mark(pl, st, "k_f32_shadow_in");
-    if (side) {
-        cudaEventRecord(pl->f32_fork, st);
-        cudaStreamWaitEvent(pl->f32_side, pl->f32_fork, 0);
-        const size_t smem = (size_t)kF32BandStage * sizeof(float);
-        cudaFuncSetAttribute(k_f32_band_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_f32_band_pass<<<(unsigned)(nf - n8), 32, smem, pl->f32_side>>>(sl + n8, pl->d_f32_items.p, pl->d_blocks.p,
-                                                                        pl->d_shadow_il.p, info,
-                                                                        (float)pl->fp32_pivot_floor);
-        launch_f32_l21(pl, blocks, info, pl->f32_side, true);
-        cudaEventRecord(pl->f32_join, pl->f32_side);
-    }
     if (nf > 0 && !hi_only) {
         if (pl->narrow_pref[SYMPIX_PREC_FP32] == 2) {  // band pass, then the border rows by column chunks
             const size_t smem = (size_t)kF32BandStage * sizeof(float);
@@ -239,16 +213,32 @@ void launch_f32_slices(sympix_plan_t pl, double *blocks, int32_t *info, cudaStre
             trace_mark(pl, st, "k_f32_band_pass");
             launch_f32_l21(pl, blocks, info, st);
         } else if (pl->narrow_pref[SYMPIX_PREC_FP32] == 3 && f32_split_fits(pl)) {
-            if (nf > n8 && !side) {
+            // w <= 8: band and border passes in separate CTAs of one launch;
+            // 9 <= w <= 12 (a few slices): band pass, then the chunked border
+            // kernels, on the side stream at the same time (a second
+            // cooperative launch would wait for the first to finish)
+            const int n8 = pl->f32_slices_w8;
+            const bool side = n8 > 0 && nf > n8 && pl->f32_side;
+            cudaStream_t sh = side ? pl->f32_side : st;
+            if (side) {
+                cudaEventRecord(pl->f32_fork, st);
+                cudaStreamWaitEvent(sh, pl->f32_fork, 0);
+            }
+            if (nf > n8) {
                 const size_t smem = (size_t)kF32BandStage * sizeof(float);
                 cudaFuncSetAttribute(k_f32_band_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                k_f32_band_pass<<<(unsigned)(nf - n8), 32, smem, st>>>(sl + n8, pl->d_f32_items.p, pl->d_blocks.p,
+                k_f32_band_pass<<<(unsigned)(nf - n8), 32, smem, sh>>>(sl + n8, pl->d_f32_items.p, pl->d_blocks.p,
                                                                       pl->d_shadow_il.p, info,
                                                                       (float)pl->fp32_pivot_floor);
-                launch_f32_l21(pl, blocks, info, st, true);
+                launch_f32_l21(pl, blocks, info, sh, true);
             }
             launch_f32_split_w8(pl, blocks, info, st);
-            trace_mark(pl, st, side ? "k_f32_split_w8" : "k_f32_split");
+            if (side) trace_mark(pl, st, "k_f32_split_w8");
+            if (side) {
+                cudaEventRecord(pl->f32_join, sh);
+                cudaStreamWaitEvent(st, pl->f32_join, 0);
+            }
+            trace_mark(pl, st, "k_f32_split");
         } else {
             launch_f32_fused(pl, nf, blocks, info, st);
         }
@@ -265,17 +255,9 @@ void launch_f32_slices(sympix_plan_t pl, double *blocks, int32_t *info, cudaStre
             launch_f32_border<512>(pl, nf, ns - nf, blocks, info, st);
         trace_mark(pl, st, "k_f32_border_pass");
     }
-    if (side) {
-        launch_factor_dense(pl, SYMPIX_PREC_FP32, false, blocks, info, st);
-        write_back(pl->d_f32_split_out[0].p, pl->d_f32_split_out[0].n);
-        trace_mark(pl, st, "k_f32_out");
-        cudaStreamWaitEvent(st, pl->f32_join, 0);
-        write_back(pl->d_f32_split_out[1].p, pl->d_f32_split_out[1].n);
-        trace_mark(pl, st, "k_f32_split");
-    } else {
-        write_back(tout, nout);
-        trace_mark(pl, st, "k_f32_out");
-    }
+    k_f32_out<float><<<(unsigned)nout, 256, 0, st>>>(tout, sl, pl->d_f32_items.p, pl->d_blocks.p, info, pl->d_shadow_il.p,
+                                             pl->d_l21_il.p, blocks);
+    trace_mark(pl, st, "k_f32_out");
     // near-degenerate blocks: FP64 from the untouched FP64 input
     launch_band<ArF64>(pl, false, blocks, info, st, 1, hi_only);
     trace_mark(pl, st, "k_factor_rescue");

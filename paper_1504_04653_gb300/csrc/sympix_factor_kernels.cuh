@@ -1046,8 +1046,6 @@ void launch_window(sympix_plan_t pl, int precision, double *blocks, int32_t *inf
 void launch_window_f64(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st);
 void launch_window_df(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st);
 constexpr int kDefaultWaitLimit = 1 << 22;  // polls of a bounded device wait (about 0.3 s)
-// the dense-format blocks of such a call (but the sliding-window launch's)
-void launch_factor_dense(sympix_plan_t pl, int precision, bool dense, double *blocks, int32_t *info, cudaStream_t st);
 void launch_factor_wide_dense(sympix_plan_t pl, int precision, bool dense, double *blocks, int32_t *info,
                               cudaStream_t st);
 

@@ -650,12 +650,6 @@ void launch_factor_wide_dense(sympix_plan_t pl, int precision, bool dense, doubl
             trace_mark(pl, st, "k_factor_wide");
         }
     }
-    // (beside its side stream the FP32 factor has launched them)
-    if (!(precision == SYMPIX_PREC_FP32 && !dense && f32_side_path(pl)))
-        launch_factor_dense(pl, precision, dense, blocks, info, st);
-}
-
-void launch_factor_dense(sympix_plan_t pl, int precision, bool dense, double *blocks, int32_t *info, cudaStream_t st) {
     const int nd = (int)pl->factor_items[3].size() -
                    dense_in_window(pl, dense ? SYMPIX_STORE_DENSE : SYMPIX_STORE_PBAND, precision);
     const int ns = (int)pl->factor_items[4].size();

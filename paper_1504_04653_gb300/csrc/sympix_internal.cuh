@@ -294,8 +294,6 @@ struct sympix_plan_s {
     std::vector<F32Slice> f32_slices;
     std::vector<int2> f32_tiles;  // (slice, first element) of the band shadow transposes
     std::vector<int2> f32_out_tiles;  // the same, then (slice, -1 - first element) of L21
-    // the write-back's tiles beside the split launch: [0] the others, [1] 9 <= w <= 12
-    sympix::DevBuf<int2> d_f32_split_out[2];
     int f32_slices_fused = 0;     // slices with w <= 12, band and border fused (they come first)
     int f32_slices_w8 = 0;        // of those, the slices with w <= 8 (they come first)
     // border rows of the fused-range slices by column chunks: work items
@@ -312,7 +310,6 @@ struct sympix_plan_s {
     // the split FP32 factor: per fused-range slice a progress and a done word
     // (zero between launches) and the band passes' results
     sympix::DevBuf<int> d_split_flags, d_split_bandres;
-    bool f32_split_ok = false;        // f32_split_fits on the plan's device
     cudaStream_t f32_side = nullptr;  // the fused 9 <= w <= 12 slices beside the w <= 8 ones
     cudaEvent_t f32_fork = nullptr, f32_join = nullptr;
     // the f32 transposes of slices with w > 12 only (the narrow-band factor
@@ -437,10 +434,4 @@ struct sympix_plan_s {
 // sliding-window launch of a factor call takes along.
 inline int dense_in_window(sympix_plan_t pl, int storage, int precision) {
     return storage == SYMPIX_STORE_PBAND && pl->narrow_pref[precision] == sympix::kNarrowWindow ? pl->win_dense : 0;
-}
-
-// Whether the FP32 factor runs its 9 <= w <= 12 slices on the side stream.
-inline bool f32_side_path(sympix_plan_t pl) {
-    return pl->narrow_pref[SYMPIX_PREC_FP32] == 3 && pl->f32_slices_w8 > 0 && pl->f32_slices_fused > pl->f32_slices_w8 &&
-           pl->f32_side && pl->f32_split_ok;
 }

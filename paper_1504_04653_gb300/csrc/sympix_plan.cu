@@ -523,20 +523,11 @@ extern "C" int sympix_support(sympix_grid_t grid, int nops, const double *r_s, i
         pl->size_l21_il = l21;
         pl->f32_out_tiles = pl->f32_tiles;
         pl->f32_out_tiles.insert(pl->f32_out_tiles.end(), tiles21.begin(), tiles21.end());
-        // the write-back of the slices of 9 <= w <= 12 apart from the others' (side stream)
-        std::vector<int2> part[2];
-        for (const int2 &t : pl->f32_out_tiles) {
-            const int w = pl->f32_slices[t.x].w;
-            part[w > 8 && w <= 12].push_back(t);
-        }
-        for (int k = 0; k < 2; ++k)
-            if ((rc = pl->d_f32_split_out[k].upload(part[k]))) return fail(rc);
         pl->f32_out_tiles_hi = pl->f32_tiles_hi;
         pl->f32_out_tiles_hi.insert(pl->f32_out_tiles_hi.end(), tiles21_hi.begin(), tiles21_hi.end());
         pl->f32_out_tiles_lo = pl->f32_tiles_lo;
         pl->f32_out_tiles_lo.insert(pl->f32_out_tiles_lo.end(), tiles21_lo.begin(), tiles21_lo.end());
     }
-    pl->f32_split_ok = f32_split_fits(pl);
     if (cudaEventCreateWithFlags(&pl->chol_fork, cudaEventDisableTiming) != cudaSuccess)
         return fail(set_error(SYMPIX_ECUDA, "sympix_support: event of the narrow-band factor"));
     if (pl->f32_slices_w8 > 0 && pl->f32_slices_fused > pl->f32_slices_w8 &&
@@ -939,8 +930,6 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
             const int n8 = pl->f32_slices_w8;
             const int nhi_items = (int)pl->l21_items.size() - pl->l21_items_w8;
             if (pl->narrow_pref[SYMPIX_PREC_FP32] == 3 && f32_split_fits(pl))
-                f += f32_side_path(pl) ? 1 : 0;  // the write-back in two parts
-            if (pl->narrow_pref[SYMPIX_PREC_FP32] == 3 && f32_split_fits(pl))
                 // the split launch (w <= 8); band pass and the five chunked kernels of 9 <= w <= 12
                 f += 2 + (n8 > 0 ? 1 : 0) + (nfu > n8 ? 1 + (nhi_items > 0 ? 5 : 0) : 0) + (nsl > nfu ? 2 : 0);
             else if (pl->narrow_pref[SYMPIX_PREC_FP32] == 2)  // band pass, then transfer, carry, solve, corner sums, corners
@@ -1041,7 +1030,6 @@ extern "C" int sympix_plan_device_bytes(sympix_plan_t pl, size_t *bytes, size_t 
         b += kv.second.d_arcs.bytes() + kv.second.d_rest.bytes() + kv.second.d_tile0.bytes() + kv.second.d_first.bytes();
     b += pl->d_apply_items.bytes() + pl->d_apply_rest.bytes() + pl->d_win_items.bytes() +
          pl->d_slot_perm.bytes() + pl->d_slot_need.bytes() + pl->d_op_order.bytes();
-    for (int i = 0; i < 2; ++i) b += pl->d_f32_split_out[i].bytes();
     for (int i = 0; i < 2; ++i) b += pl->d_win[i].bytes() + pl->d_apply_work[i].bytes();
     for (int i = 0; i < 5; ++i) b += pl->d_items_pband[i].bytes();
     for (int i = 0; i < 3; ++i) b += pl->d_items_wide[i].bytes();
