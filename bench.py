@@ -56,9 +56,10 @@ def parse(argv=None):
                     help="replay the step as captured CUDA graphs, or call the entry points directly")
     ap.add_argument("--no-autotune", action="store_true", help="keep the default launch shapes")
     ap.add_argument("--narrow-factor", type=int, default=None, choices=[-1, 0, 1, 2, 3],
-                    help="kernel for bands w <= 12: 0 G-lane, 1 earlier kernels, 2 band pass and chunked "
-                         "border on a shadow of the arithmetic, 3 FP32 split CTAs, -1 per arithmetic (default: "
-                         "the autotuner's choice)")
+                    help="kernel for bands w <= 12: 0 G-lane, 1 earlier kernels, 2 sliding window (FP32: "
+                         "band pass and chunked border on a shadow), 3 band pass and chunked border on a shadow "
+                         "of the arithmetic (FP32: split CTAs), -1 per arithmetic (default: the autotuner's "
+                         "choice)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-configs", action="store_true", help="skip the l_max 1500 and 32-operator sub-lines")
@@ -305,12 +306,12 @@ def kernel_models(plan, grid, sprec, fprec):
     # remainder after it ("k_f32_split"), which is not a kernel's own time
     m.update({"k_f32_split_w8": (b8, fl8, "fp32"), "k_f32_fused_w8": (b8, fl8, "fp32"),
               "k_f32_split": (0.0, None, "fp32", "the w 9..12 path's time beyond the w <= 8 launch, not a kernel")})
-    # option 2 (band pass of every slice, border rows by column chunks): its
+    # the chunked border (band pass of every slice, border rows by column chunks): its
     # chunk kernels are not modelled separately
     for name in ("k_l21_transfer", "k_l21_carry", "k_l21_solve", "k_l21_cornerpart", "k_l21_corner"):
         m[name] = (0.0, None, "fp32", "a phase of the chunked border solve, not modelled alone")
     if fprec in ("fp64", "fp32x2"):
-        # FP64 / split FP32 on a shadow of 8-byte elements (option 2, w <= 12):
+        # FP64 / split FP32 on a shadow of 8-byte elements (option 3, w <= 12):
         # the transposes move 16 B per element (FP64 read or written, the
         # shadow element written or read), the band pass reads and writes its
         # rows (16 B) and does the band third of the factor's flops

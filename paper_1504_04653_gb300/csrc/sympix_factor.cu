@@ -63,9 +63,9 @@ extern "C" int sympix_factor_blocks(sympix_plan_t pl, int storage, int precision
     if (narrow) launch_pband_chol(pl, precision, blocks, info, st);
     if (precision != SYMPIX_PREC_FP32 && !dense && pl->narrow_pref[precision] == kNarrowWindow) {
         launch_window(pl, precision, blocks, info, st);  // w <= 12 in one pass, lane groups above
-    } else if (precision == SYMPIX_PREC_FP64 && !dense && pl->narrow_pref[precision] == 2) {
+    } else if (precision == SYMPIX_PREC_FP64 && !dense && pl->narrow_pref[precision] == kNarrowChunked) {
         launch_f64_slices(pl, blocks, info, st);  // w <= 12 on the FP64 shadow, lane groups above
-    } else if (precision == SYMPIX_PREC_FP32X2 && !dense && pl->narrow_pref[precision] == 2) {
+    } else if (precision == SYMPIX_PREC_FP32X2 && !dense && pl->narrow_pref[precision] == kNarrowChunked) {
         launch_df_slices(pl, blocks, info, st);  // w <= 12 on a split-FP32 shadow, lane groups above
     } else if (precision == SYMPIX_PREC_FP64) {
         if (!narrow) launch_band<ArF64>(pl, dense, blocks, info, st);  // (narrow: every w <= 16 done)

@@ -59,8 +59,9 @@ bool f32_split_fits(sympix_plan_t pl);
 // Widest band of the narrow-band factor (k_pband_chol), and the elements of
 // one tile of its FP32 commit.
 constexpr int kNarrowWMax = 12;
-// narrow_pref of the sliding-window kernel (FP64 and split FP32)
-constexpr int kNarrowWindow = 4;
+// narrow_pref of FP64 and split FP32: the sliding-window kernel, and the band
+// pass with the chunked border solve
+constexpr int kNarrowWindow = 2, kNarrowChunked = 3;
 constexpr int kCommitTileElems = 2048;
 
 // Smallest relative distance |u - u_s| / u_s a support class may have from
@@ -345,9 +346,10 @@ struct sympix_plan_s {
     // kernel for periodic bands w <= 12, per factor arithmetic (SYMPIX_PREC_*):
     // 0 k_pband_chol (G lanes per block), 1 the earlier kernels (FP32: the
     // two-role kernel on an FP32 band copy; FP64 / split FP32: lane groups),
-    // 2 band pass and chunked border solve on a shadow of the arithmetic,
-    // 3 (FP32) band and border CTAs of one cooperative launch for w <= 8, 2
-    // for 9 <= w <= 12, kNarrowWindow (FP64 and split FP32) the sliding window.
+    // 2 the sliding window (FP32: band pass and chunked border solve on a
+    // shadow), 3 that band pass and border solve on a shadow of the arithmetic
+    // (FP32: band and border CTAs of one cooperative launch for w <= 8, 2 for
+    // 9 <= w <= 12)
     int narrow_pref[3] = {sympix::kNarrowWindow, 3, sympix::kNarrowWindow};
     // DP-grid plans (k > 1): band blocks under tile adjacency
     bool tiles = false;
@@ -433,5 +435,8 @@ struct sympix_plan_s {
 // The small dense-format blocks (the last of factor_items[3]) that the
 // sliding-window launch of a factor call takes along.
 inline int dense_in_window(sympix_plan_t pl, int storage, int precision) {
-    return storage == SYMPIX_STORE_PBAND && pl->narrow_pref[precision] == sympix::kNarrowWindow ? pl->win_dense : 0;
+    return storage == SYMPIX_STORE_PBAND && precision != SYMPIX_PREC_FP32 &&
+                   pl->narrow_pref[precision] == sympix::kNarrowWindow
+               ? pl->win_dense
+               : 0;
 }

@@ -716,11 +716,6 @@ extern "C" int sympix_plan_option(sympix_plan_t pl, int option, double value) {
             pl->narrow_pref[SYMPIX_PREC_FP64] = kNarrowWindow;
             pl->narrow_pref[SYMPIX_PREC_FP32] = 3;
             pl->narrow_pref[SYMPIX_PREC_FP32X2] = kNarrowWindow;
-        } else if (value == 2.0 || value == 3.0) {
-            // the chunked border solve (every arithmetic) and the split kernel (FP32)
-            pl->narrow_pref[SYMPIX_PREC_FP64] = 2;
-            pl->narrow_pref[SYMPIX_PREC_FP32] = (int)value;
-            pl->narrow_pref[SYMPIX_PREC_FP32X2] = 2;
         } else {
             for (int &v : pl->narrow_pref) v = (int)value;
         }
@@ -761,7 +756,7 @@ extern "C" int sympix_plan_tuning(sympix_plan_t pl, int *table_cta, int *border_
     if (table_cta) *table_cta = pl->table_cta;
     if (border_threads) *border_threads = pl->border_threads;
     if (narrow)
-        for (int i = 0; i < 3; ++i) narrow[i] = pl->narrow_pref[i] == kNarrowWindow ? 2 : pl->narrow_pref[i];
+        for (int i = 0; i < 3; ++i) narrow[i] = pl->narrow_pref[i];
     return SYMPIX_OK;
 }
 
@@ -808,8 +803,7 @@ extern "C" int sympix_autotune(sympix_plan_t pl, const double *bl, const double 
         factor_precision <= 2) {
         best = 1e30f;
         int best_k = pl->narrow_pref[factor_precision];
-        for (int kk : {0, 1, 2, 3, kNarrowWindow}) {
-            if (kk == (factor_precision == SYMPIX_PREC_FP32 ? kNarrowWindow : 3)) continue;
+        for (int kk : {0, 1, 2, 3}) {
             pl->narrow_pref[factor_precision] = kk;
             float ms = 0.0f;
             auto run = [&] {
@@ -946,7 +940,7 @@ extern "C" int sympix_plan_launches(sympix_plan_t pl, int storage, int sample_pr
     } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == kNarrowWindow) {
         // w <= 12 in the sliding-window kernel, then the lane groups of 12 < w <= 16
         f += (pl->d_win[0].n > 0 ? 1 : 0) + (l2 ? 1 : 0);
-    } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == 2) {
+    } else if (factor_precision != SYMPIX_PREC_FP32 && pband && pl->narrow_pref[factor_precision] == kNarrowChunked) {
         // w <= 12 on the FP64 / split-FP32 shadow: transpose in, band pass, transfer, carry,
         // solve and corner sums of each width range, corners, write-back; then
         // the lane groups of 12 < w <= 16

@@ -35,7 +35,7 @@
 // its warp, whatever the number of active lanes (measured; 76 with the other
 // three schedulers busy).  At W = 8 a step has 5 of them for the root, 1 for t,
 // W (or W/2 with one block per warp) updates and W(W+1)/2G for the corner.
-// One block per lane (the band pass of option 2) spends fewer instructions per
+// One block per lane (the band pass of option 3) spends fewer instructions per
 // block, but its step takes 1.8k cycles and the border needs a second pass of
 // about the same length; here a block's n steps take 1210 cycles each in FP64
 // and 780 in split FP32 for band and border together, and nothing is

@@ -223,7 +223,8 @@ class Plan:
         return a.value, b.value
 
     def narrow_kernels(self):
-        """{arithmetic: 0 (G-lane), 1 (earlier kernels), 2 (FP32 chunked border) or 3 (FP32 split CTAs)}."""
+        """{arithmetic: 0 (G-lane), 1 (earlier kernels), 2 (sliding window; FP32 chunked border) or
+        3 (chunked border; FP32 split CTAs)}: what set_narrow_factor selects."""
         nk = (ctypes.c_int * 3)()
         _check(lib().sympix_plan_tuning(self._h, None, None, nk))
         return {"fp64": nk[0], "fp32": nk[1], "fp32x2": nk[2]}
@@ -237,9 +238,9 @@ class Plan:
         return self.tuning()
 
     def set_narrow_factor(self, kernel: int):
-        """w <= 12 bands: 0 the G-lane kernel, 1 the earlier kernels, 2 (every arithmetic) the band
-        pass and the border rows by column chunks, 3 (FP32; the others as 2) band and border passes in
-        two CTAs of one cooperative launch, -1 per arithmetic (default)."""
+        """w <= 12 bands: 0 the G-lane kernel, 1 the earlier kernels, 2 the sliding window (FP32: the
+        band pass and the border rows by column chunks), 3 that band pass and chunked border (FP32: band
+        and border passes in two CTAs of one cooperative launch), -1 per arithmetic (default)."""
         _check(lib().sympix_plan_option(self._h, OPT_NARROW_FACTOR, float(kernel)))
 
     def set_wait_limit(self, polls: int):
