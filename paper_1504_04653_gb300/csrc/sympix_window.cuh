@@ -525,11 +525,7 @@ __device__ __forceinline__ void window_dense(const BlockDesc *__restrict__ block
 // of its SM: CTAs of one warp were placed unevenly (up to three on one
 // scheduler and none on another), which doubled the time.
 constexpr int kWindowWarps = 4;
-// Shared memory that keeps a third CTA off the SM: the longest blocks set the
-// time and come first, and a third warp on each scheduler slows them down
-// (l_max 3000 FP64 8.7 ms with three, 7.5 ms with two).
-constexpr int kWindowSmemMin = 80 * 1024;
-
+// (two CTAs per SM: the registers allow no more)
 template <class V, bool ONE>
 __global__ void __launch_bounds__(32 * kWindowWarps, 2) k_window_chol(int count, int smem_warp,
                                                                    const int4 *__restrict__ work,
@@ -557,12 +553,12 @@ __global__ void __launch_bounds__(32 * kWindowWarps, 2) k_window_chol(int count,
 
 template <class V, bool ONE>
 void launch_window_list(sympix_plan_t pl, double *blocks, int32_t *info, cudaStream_t st) {
-    size_t smem = pl->win_dense ? 32 * 33 * sizeof(double) : 16;
-    for (int w = 1; w <= pl->chol_wmax; ++w) {
+    // one size for every plan: the limit is the function's, not a launch's
+    size_t smem = 32 * 33 * sizeof(double);  // a small dense block
+    for (int w = 1; w <= kNarrowWMax; ++w) {
         const int g = ONE ? 32 : window_rows(w);
         smem = std::max(smem, (size_t)(32 / g) * window_elems(w, g) * 8);
     }
-    smem = std::max(smem, (size_t)kWindowSmemMin / kWindowWarps);
     const int count = (int)pl->d_win[ONE].n;
     cudaFuncSetAttribute(k_window_chol<V, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(kWindowWarps * smem));
