@@ -475,15 +475,22 @@ __global__ void __launch_bounds__(32) k_apply(const int32_t *__restrict__ items,
     for (int c = lane; c < n; c += 32) yout[c * ps] = v[c];
 }
 
-// Dynamic shared memory of one warp of k_apply_band.
+// Dynamic shared memory of one warp of k_apply_band on entries of width w, of
+// the plan's widest entry, and of any.
+static size_t apply_smem_width(int w, bool one) {
+    const int g = one ? 32 : apply_lanes(w);
+    const size_t e = w < 0 ? 32 * 33 : w == 0 ? 2 : (size_t)(32 / g) * apply_elems(w);
+    return (e * sizeof(double) + 15) / 16 * 16;
+}
 static size_t apply_smem(sympix_plan_t pl, bool one) {
     size_t smem = 16;
-    for (const int4 &it : pl->apply_work[one]) {
-        const int g = one ? 32 : apply_lanes(it.z);
-        const size_t e = it.z < 0 ? 32 * 33 : it.z == 0 ? 2 : (size_t)(32 / g) * apply_elems(it.z);
-        smem = std::max(smem, e * sizeof(double));
-    }
-    return (smem + 15) / 16 * 16;
+    for (const int4 &it : pl->apply_work[one]) smem = std::max(smem, apply_smem_width(it.z, one));
+    return smem;
+}
+static size_t apply_smem_max(bool one) {
+    size_t smem = 16;
+    for (int w = -1; w <= kApplyWMax; ++w) smem = std::max(smem, apply_smem_width(w, one));
+    return smem;
 }
 
 template <bool ONE>
@@ -492,7 +499,10 @@ static void launch_apply_band(sympix_plan_t pl, const double *blocks, const int3
     const int count = (int)pl->apply_work[ONE].size();
     if (!count) return;
     const size_t smem = apply_smem(pl, ONE);
-    cudaFuncSetAttribute(k_apply_band<ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kApplyWarps * smem));
+    // the limit is the function's, not a launch's: the same for every plan,
+    // whatever other threads and captured graphs launch
+    cudaFuncSetAttribute(k_apply_band<ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kApplyWarps * apply_smem_max(ONE)));
     k_apply_band<ONE><<<(unsigned)((count + kApplyWarps - 1) / kApplyWarps), 32 * kApplyWarps, kApplyWarps * smem, st>>>(
         count, (int)smem, pl->d_apply_work[ONE].p, pl->d_apply_items.p, pl->d_blocks.p, info, blocks, pl->d_ring_off.p,
         pl->d_ring_stride.p, pl->grid->npix, x, y);
@@ -566,7 +576,7 @@ extern "C" int sympix_apply(sympix_plan_t pl, int storage, const double *blocks,
         // reciprocal diagonals (the widest periodic band planned)
         const size_t W1 = (size_t)pl->max_w + 1;
         const size_t smem = ((size_t)pl->grid->max_ring + (kApplyRows + W1) * (W1 + 1)) * sizeof(double);
-        cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);  // what a CTA may have
         k_apply<<<(unsigned)nrest, 32, smem, st>>>(band ? pl->d_apply_rest.p : nullptr, pl->d_blocks.p, info, blocks,
                                                    storage == SYMPIX_STORE_DENSE ? 1 : 0, pl->d_ring_off.p,
                                                    pl->d_ring_stride.p, pl->grid->npix, pl->grid->max_ring, x, y);

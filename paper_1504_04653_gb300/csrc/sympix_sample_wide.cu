@@ -275,8 +275,7 @@ static void launch_wide32(sympix_plan_t pl, int list, double *blocks, cudaStream
     if (pl->items_wide[list].empty()) return;
     const int w = pl->wide_list_w[list];
     const size_t staged = kWideRings * (size_t)(kWideMap + kWideTab), walked = (size_t)(w + 1 + wide_arc(w)) * kWalkCols;
-    const size_t smem = std::max(staged, walked) * sizeof(float);
-    cudaFuncSetAttribute(k_sample_wide32<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = std::max(staged, walked) * sizeof(float);  // at most 37 KB: no limit to raise
     k_sample_wide32<NT><<<(unsigned)pl->items_wide[list].size(), NT, smem, st>>>(
         pl->d_items_wide[list].p, pl->d_blocks.p, pl->d_entries.p, pl->nslots, pl->grid->npix, pl->d_tab_b32.p,
         pl->d_tab_d32.p, pl->d_ninv32.p, blocks);
