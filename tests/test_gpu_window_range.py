@@ -1,4 +1,4 @@
-"""The split-FP32 sliding-window factor (w <= 12) over the FP32 range: blocks
+"""The sliding-window factor (w <= 12) over the range of its arithmetic: blocks
 scaled as a whole and row by row, against the backward error of Cholesky."""
 import numpy as np
 import pytest
@@ -76,3 +76,43 @@ def test_scaled_blocks(reps, rows, top):
         widths.add(int(w))
     print(f"top {top} rows {rows}: worst error / bound {worst:.3g}")
     assert len(widths) >= 6 and {2, 4, 8} <= widths and max(widths) >= 10, sorted(widths)
+
+
+@pytest.mark.parametrize("reps", [1, 3])
+@pytest.mark.parametrize("top", [-1040, -1000, 0, 1000, 1022])
+def test_scaled_blocks_fp64(reps, top):
+    """The same in FP64, down into the subnormal numbers, which lose what lies
+    below 2^-1074: |L L^T - M|_ij <= 8 (2w + 2) (2^-53 s_ij + 2^-1074).  Every
+    well-conditioned block factors, in every width from 0 to 12."""
+    import torch
+    from paper_1504_04653_gb300 import sympix as S
+    grid, plan, host = _blocks(S, reps)
+    picked = {}
+    for o in range(plan.nops):
+        for j in range(grid.nrings):
+            off, n, w, fmt = plan.block_layout("pband", o, j)
+            if fmt != S.BLOCK_PBAND or w > 12:
+                continue
+            rowsview = host[off:off + n * (w + 1)].reshape(n, w + 1)
+            big = int(np.floor(np.log2(rowsview[:, 0].max())))
+            half = (top - big) // 2
+            rowsview *= 2.0 ** half
+            rowsview *= 2.0 ** half
+            if not (o >= len(RADII) and (o + j) % 5) and j % 2 == 0:
+                picked[o, j] = (n, w)
+    blocks = torch.tensor(host).cuda()
+    info = S.sympix_factor_blocks(plan, blocks, precision="fp64").cpu().numpy()
+    got, widths = blocks.cpu().numpy(), set()
+    up = 2.0 ** (-(top // 2))  # both sides back to where numpy's products are normal numbers
+    for (o, j), (n, w) in picked.items():
+        M = S.unpack_block(host, plan, "pband", o, j) * up * up
+        diag = np.sqrt(np.diag(M))
+        if np.linalg.eigvalsh(M / diag / diag[:, None])[0] < 1e-3:
+            continue
+        assert info[o * grid.nrings + j] == 0, (o, j, n, w, int(info[o * grid.nrings + j]))
+        L = S.unpack_block(got, plan, "pband", o, j, factored=True) * up
+        bound = 8 * (2 * w + 2) * (2.0 ** -53 * diag * diag[:, None] + 2.0 ** -1074 * up * up)
+        assert np.max(np.abs(L @ L.T - M) / bound) <= 1.0, (o, j, n, w, np.max(np.abs(L @ L.T - M) / bound))
+        widths.add(int(w))
+    print(sorted(widths))
+    assert {0, 2, 4, 6, 8, 10, 12} <= widths, sorted(widths)
